@@ -1095,9 +1095,12 @@ struct BoxView {
 // memory, with 256 or 512 threads per brick; or fixed-point atomics into an L2-resident
 // scratch) give the same delta' bit for bit, so the choice changes only the speed.  Each
 // candidate allowed by params.deposit_form is timed with CUDA events on this context's own
-// boxes (one box in the per-tile form), with the particles where C.1-C.3 put them, and the
-// fastest is kept for the life of the context and for its captured graph.  Runs once,
-// before the first capture; needs the boxes set up (it launches C.1-C.3 itself).
+// boxes (one box in the per-tile form), with the particles where the LPT of the run puts them at
+// the middle force evaluation (on the initial lattice, where neighbours share cells, the
+// atomics look faster than they are over a run: 0.64 ms against 0.98 ms at a = 1 on 64 boxes of
+// 72-96 cells, one per particle), and the fastest is kept for the life of the context and for
+// its captured graph.  Runs once, before the first capture; needs the LPT fields (it launches
+// C.1-C.3 itself).
 scola_status autotune_deposit(scola_ctx *c) {
     if (c->tuned) return SCOLA_OK;
     struct Cand {
@@ -1113,10 +1116,11 @@ scola_status autotune_deposit(scola_ctx *c) {
     {
         std::unique_ptr<BoxView> view;
         if (c->prm.batch_mode == SCOLA_BATCH_PER_TILE) view.reset(new BoxView(c, 0));
-        CK(launch_box_init(*c));
+        const size_t mid = c->tt.D1.size() / 2;
+        CK(launch_box_init(*c, c->tt.D1[mid], c->tt.D2[mid]));
         CK(launch_shell(*c));
         CK(launch_pad(*c, 1.0f));
-        const float inv_D1 = (float)(1.0 / c->tt.D1[0]);
+        const float inv_D1 = (float)(1.0 / c->tt.D1[mid]);
         for (int q = lo; q < hi; ++q) {
             c->deposit_form = all[q].form;
             c->deposit_threads = all[q].threads;
@@ -1230,7 +1234,7 @@ scola_status enqueue_evolution_per_tile(scola_ctx *c) {
     const int n = (int)c->tt.alpha.size();
     for (int b = 0; b < c->nboxes; ++b) {
         BoxView v(c, b);
-        CK(launch_box_init(*c));
+        CK(launch_box_init(*c, c->tt.D1_i, c->tt.D2_i));
         CK(launch_shell(*c));
         CK(launch_pad(*c, 1.0f));
         for (int k = 0; k <= n; ++k) {
@@ -1250,7 +1254,7 @@ scola_status enqueue_evolution_per_tile(scola_ctx *c) {
 // force evaluation.
 scola_status enqueue_evolution(scola_ctx *c) {
     if (c->prm.batch_mode == SCOLA_BATCH_PER_TILE) return enqueue_evolution_per_tile(c);
-    CK(launch_box_init(*c));
+    CK(launch_box_init(*c, c->tt.D1_i, c->tt.D2_i));
     CK(launch_shell(*c));
     CK(launch_pad(*c, 1.0f));
     const int n = (int)c->tt.alpha.size();
@@ -1538,7 +1542,7 @@ scola_status scola_setup_boxes(scola_ctx *c) {
     CS(autotune_deposit(c));
     CS(autotune_dst(c));
     c->have_forward = false;            // the particle state of the last forward run is replaced
-    CK(launch_box_init(*c));
+    CK(launch_box_init(*c, c->tt.D1_i, c->tt.D2_i));
     CK(launch_shell(*c));
     CK(launch_pad(*c, 1.0f));
     c->setup_done = true;

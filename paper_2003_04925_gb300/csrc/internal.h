@@ -238,7 +238,7 @@ cudaError_t launch_source_init(Ctx &c, const float *xx, const float *yy, const f
 cudaError_t launch_source_sub(Ctx &c, const float *t, float *S);
 cudaError_t launch_gradient(Ctx &c, const float *phi, float *psi);
 
-cudaError_t launch_box_init(Ctx &c);
+cudaError_t launch_box_init(Ctx &c, double D1, double D2);   // s = -D1 Psi1 + D2 Psi2, p_res = 0
 cudaError_t launch_shell(Ctx &c);
 // Ghost layers of the padded potential <- D1 x shell.  The solve runs on Phi / D1(a_K), so
 // the ghost layers hold the unscaled shell (D1 = 1), written once per forward run.

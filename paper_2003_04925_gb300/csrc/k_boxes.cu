@@ -224,11 +224,10 @@ int grid_for(long long n, int block) {
 
 }  // namespace
 
-cudaError_t launch_box_init(Ctx &c) {
+cudaError_t launch_box_init(Ctx &c, double D1, double D2) {
     const int Ntile = c.Np / c.Ntiles;
     k_box_init<<<c.n_pchunks, kChunk, 0, c.stream>>>(c.boxes, c.pchunks, c.part, c.P, c.psi1, c.psi2,
-                                                      c.Np, Ntile, c.N3, (float)c.tt.D1_i,
-                                                      (float)c.tt.D2_i);
+                                                      c.Np, Ntile, c.N3, (float)D1, (float)D2);
     ++c.launches;
     return cudaGetLastError();
 }

@@ -216,6 +216,45 @@ __device__ __forceinline__ void deposit_entry(unsigned long long *acc, const flo
     }
 }
 
+// The same for an entry whose eight corners all lie in the brick and the mesh (class 0 of a
+// full brick): no bounds checks, and the 2^32 scale folded into the z weights (an exact power
+// of two, so every product is the one of weight_to_fixed).  A weight of exactly 1 (a particle on
+// a cell centre) does not fit 32 bits: such entries take the checked form.
+template <int kMode>
+__device__ __forceinline__ void deposit_inside(unsigned long long *acc, const float4 v, int x0, int y0, int z0) {
+    const int pk = __float_as_int(v.w);
+    const int cell = ((((pk & 1023) - 2 - x0) * kBrick) + (((pk >> 10) & 1023) - 2 - y0)) * kBrick +
+                     (((pk >> 20) & 1023) - 2 - z0);
+    const float wx[2] = {1.0f - v.x, v.x}, wy[2] = {1.0f - v.y, v.y};
+    const float wz[2] = {(1.0f - v.z) * 4294967296.0f, v.z * 4294967296.0f};
+    unsigned *lo = reinterpret_cast<unsigned *>(acc) + cell, *hi = lo + kBrickCells;
+#pragma unroll
+    for (int ex = 0; ex < 2; ++ex)
+#pragma unroll
+        for (int ey = 0; ey < 2; ++ey) {
+            const float wxy = wx[ex] * wy[ey];
+#pragma unroll
+            for (int ez = 0; ez < 2; ++ez) {
+                const int c = (ex * kBrick + ey) * kBrick + ez;
+                const unsigned f = __float2uint_rn(wxy * wz[ez]);
+                if (kMode == kAccHalves) {
+                    const unsigned old = atomicAdd(lo + c, f);
+                    if (old > ~f) atomicAdd(hi + c, 1u);          // the low half wrapped
+                } else if (kMode == kAccRed16) {
+                    atomicAdd(lo + c, f & 0xffffu);
+                    atomicAdd(hi + c, f >> 16);
+                } else {
+                    atomicAdd(acc + cell + c, (unsigned long long)f);
+                }
+            }
+        }
+}
+
+// Whether some corner weight of the entry is exactly 1.
+__device__ __forceinline__ bool unit_weight(const float4 v) {
+    return fmaxf(v.x, 1.0f - v.x) == 1.0f && fmaxf(v.y, 1.0f - v.y) == 1.0f && fmaxf(v.z, 1.0f - v.z) == 1.0f;
+}
+
 // One CTA of T threads per real brick (item.start = brick index in the box, nb^3 of them).
 // kMode: the counter form (kAcc64, kAccHalves, kAccRed16).
 template <int kBrickThreads, int kMode>
@@ -273,12 +312,19 @@ k_sort_brick(const BoxDesc *__restrict__ boxes, const Chunk *__restrict__ items,
             else deposit_entry<kMode, false>(acc, v, x0, y0, z0, Ng);
         }
     };
+    // entries of class 0 (the first slice: no corner in a lower brick) of a full brick have every
+    // corner inside: 82 % of the entries of a smooth field, at half the instructions of the rest
+    const int inner = full && (kMode != kAccRed16 || red16) ? seg_start[1] : 0;
+    auto deposit_own = [&](const float4 &v, int e) {
+        if (e < inner && !unit_weight(v)) deposit_inside<kMode>(acc, v, x0, y0, z0);
+        else deposit(v);
+    };
     for (int e = tid; e < own; e += 2 * kBrickThreads) {
         const bool two = e + kBrickThreads < own;
         const float4 v0 = own_list[e];
         const float4 v1 = two ? own_list[e + kBrickThreads] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        deposit(v0);
-        if (two) deposit(v1);
+        deposit_own(v0, e);
+        if (two) deposit_own(v1, e + kBrickThreads);
     }
     for (int e = own + tid; e < total; e += kBrickThreads) {
         int lo = 8, hi = kSegments;              // seg_start[lo] <= e < seg_start[hi]
