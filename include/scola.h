@@ -52,23 +52,29 @@ typedef enum scola_status {
 } scola_status;
 
 typedef enum scola_dst_variant {
-    SCOLA_DST_SIMT = 0,          /* dense sine-matrix pencils on FP32 CUDA cores */
+    SCOLA_DST_SIMT = 0,          /* dense sine-matrix products on FP32 CUDA cores; at FDA order 2 and
+                                    Ng <= 128 whole x planes in shared memory (z and y in one pass)
+                                    and elimination along x */
     SCOLA_DST_TC_3XTF32 = 1,     /* the same products on tcgen05 tensor cores, 3xTF32 split;
                                     every 2 <= Ng <= 240 (the sine matrix resident in shared
-                                    memory, folded by its mirror symmetry for Ng > 128) */
+                                    memory, folded by its mirror symmetry for Ng > 128).  At FDA
+                                    order 2 the x axis is solved by elimination: with z and y in
+                                    sine space the Laplacian is tridiagonal along x */
     SCOLA_DST_TC_4XTF32 = 3,     /* as 1, plus the lo x lo product (four TF32 products) */
-    SCOLA_DST_TC_3PASS = 4,      /* the products in three mesh passes instead of six: z forward
-                                    (3xTF32); every z-frequency plane transformed along y and x,
-                                    divided and transformed back in shared memory (3xFP16, each
-                                    pencil scaled by a power of two into FP16's range: the same
-                                    ~22 bits as 3xTF32 at twice its rate); z inverse (3xTF32).
-                                    Every Ng <= 96 with Ng % 4 == 0 (UNSUPPORTED otherwise) */
+    SCOLA_DST_TC_3PASS = 4,      /* the products in three mesh passes instead of one per axis.  FDA
+                                    order 2: every x plane transformed along z and y in shared
+                                    memory, elimination along x, every x plane transformed back.
+                                    Orders 4 and 6: z forward; every z-frequency plane transformed
+                                    along y and x, divided and transformed back; z inverse.  The
+                                    plane products are 3xFP16, each pencil scaled by a power of two
+                                    into FP16's range: the same ~22 bits as 3xTF32 at twice its
+                                    rate.  Every Ng <= 96 with Ng % 4 == 0 (UNSUPPORTED otherwise) */
     SCOLA_DST_RADIX = 5,         /* fast sine transforms on FP32 CUDA cores, O(Ng log Ng) per
                                     pencil: each DST-I of length Ng from a real DFT of length
                                     Ng + 1 (two pencils per complex transform), done by
                                     Bluestein's chirp convolution with radix-16 FFTs of a power-of-two
                                     length in shared memory; every 1 <= Ng <= 256 */
-    SCOLA_DST_AUTO = 2           /* the fastest of the tensor-core forms (six passes, and three
+    SCOLA_DST_AUTO = 2           /* the fastest of the tensor-core forms (one axis a pass, and three passes
                                     where every Ng allows it), the dense FP32 form and the radix
                                     form, timed once on the context's boxes before the first
                                     evolution (where Ng > 222 excludes the dense FP32 form: the
@@ -207,7 +213,8 @@ typedef struct scola_stats {
     double ms_lpt;                /* initial-condition and 2LPT stage, device time (on the
                                      first call, plus the deposit autotuner's runs) */
     double ms_evolve;             /* gather + evolution + scatter, device time */
-    int64_t kernel_launches;      /* kernels launched by the last forward call */
+    int64_t kernel_launches;      /* kernels launched by the last forward call (a full-box Fourier
+                                     transform of the initial conditions counts one per axis) */
     int32_t deposit_form;         /* the form in use: SCOLA_DEPOSIT_SORTED or _ATOMIC (0 before
                                      the first scola_forward / scola_setup_boxes) */
     int32_t deposit_threads;      /* threads per brick CTA of the sorted form, else 0 */
@@ -392,10 +399,11 @@ scola_status scola_set_profiling(scola_ctx *ctx, int32_t enable);
  * forward run made in profiling mode (synchronises on it).  ms_per_launch
  * (host, n >= 8 doubles) receives, in order: deposit (with the boundary source
  * and the clearing of its counters), the Poisson passes 1..6, interpolate +
- * kick + drift.  FP32 form: pass 1 z forward, 2 y forward,
- * 3 x forward + sine-space division + x inverse, 4 y inverse, 5 z inverse,
- * 6 empty.  Tensor-core form: 1 z forward, 2 y forward, 3 x forward +
- * division, 4 z inverse, 5 y inverse, 6 x inverse.
+ * kick + drift.  Three-pass forms (and the FP32 form at Ng <= 128) at FDA order 2: 1 z and y
+ * forward, 2 elimination along x, 3 z and y inverse, the rest empty.  FP32 form otherwise: pass
+ * 1 z forward, 2 y forward, 3 x forward + sine-space division + x inverse, 4 y inverse,
+ * 5 z inverse, 6 empty.  Tensor-core form: 1 z forward, 2 y forward, 3 elimination along x,
+ * 4 z inverse, 5 y inverse, 6 empty (orders 4 and 6: 3 x forward + division, 6 x inverse).
  * Errors: STATE when profiling is off.
  */
 scola_status scola_kernel_times(const scola_ctx *ctx, double *ms_per_launch, int32_t n);

@@ -46,7 +46,6 @@ struct scola_ctx : public Ctx {
     std::vector<BoxGeom> ctx_geo;        // the context's boxes
     cudaStream_t cap_stream = nullptr;   // stream used only to capture the evolution graph
     long long graph_kernels = 0;         // kernels in the evolution graph
-    long long lpt_kernels = 0;           // kernels of the last LPT stage
     float *w_h2d = nullptr, *x_h2d = nullptr, *p_h2d = nullptr;  // buffers of scola_forward_host
     bool profiling = false;
     std::vector<cudaEvent_t> prof_ev;    // KC_COUNT + 1 events per force evaluation
@@ -72,6 +71,13 @@ struct scola_ctx : public Ctx {
             set_error(std::string(#call) + ": cuFFT error " + std::to_string((int)_r)); \
             return SCOLA_ERR_CUDA;                                                   \
         }                                                                            \
+    } while (0)
+
+// A full-box transform of the LPT stage, counted as one kernel per axis.
+#define CT(call)                                                                     \
+    do {                                                                             \
+        CF(call);                                                                    \
+        c->launches += 3;                                                            \
     } while (0)
 
 #define CS(call)                                                                     \
@@ -219,6 +225,9 @@ struct BatchPlan {
     std::vector<long long> group_plane_first;
     std::vector<int> group_nplanes, plane_beg;
     long long n_planes = 0;
+    std::vector<Chunk> tri, xpl;                       // FDA order 2: boxes by Ng; x planes
+    std::vector<int> tri_first, tri_count, tri_at, xpl_beg;
+    long long n_xpl = 0;
     std::vector<Chunk> rxt;                            // radix DST: (box, tile) per group
     long long n_rxt = 0;
     std::vector<long long> rx_group_first;
@@ -374,6 +383,25 @@ void plan_batch(const scola_ctx *c, const std::vector<BoxGeom> &tiling_geo, int 
             }
             bp.group_nplanes.push_back((int)(bp.n_planes - bp.group_plane_first.back()));
         }
+    // FDA order 2: the boxes of each Ng, and (small meshes) every x plane of each box
+    bp.tri_at.assign(count, 0);
+    for (const TriGroup &G : c->tri_groups) {
+        bp.tri_first.push_back((int)bp.tri.size());
+        for (int b = 0; b < count; ++b)
+            if (bp.geo[b].ng == G.Ng) {
+                bp.tri_at[b] = (int)bp.tri.size();
+                bp.tri.push_back({b, 0});
+            }
+        bp.tri_count.push_back((int)bp.tri.size() - bp.tri_first.back());
+    }
+    bp.xpl_beg.assign(count, 0);
+    if (small_supported(*c))
+        for (int b = 0; b < count; ++b) {
+            bp.xpl_beg[b] = (int)bp.n_xpl;
+            if (lists)
+                for (int i = 0; i < bp.geo[b].ng; ++i) bp.xpl.push_back({b, i});
+            bp.n_xpl += bp.geo[b].ng;
+        }
     // radix DST tiles: per Ng group, each box's tiles of 2 R rows
     bp.rx_tile_beg.assign(count, 0);
     bp.rx_tile_end.assign(count, 0);
@@ -474,6 +502,8 @@ scola_status bind_batch(scola_ctx *c, int k, bool force = false) {
     if (c->use_tc) CS(put(c->tc_tiles, bp.tct));
     if (c->tc3_ok) CS(put(c->tc_planes, bp.planes));
     if (c->rx_ok) CS(put(c->rx_tiles, bp.rxt));
+    CS(put(c->tri_boxes, bp.tri));
+    CS(put(c->xplanes, bp.xpl));
     c->nboxes = count;
     c->boxes_h = bp.boxes;
     c->n_pchunks = (int)bp.n_pch;
@@ -500,6 +530,13 @@ scola_status bind_batch(scola_ctx *c, int k, bool force = false) {
         c->tc_groups[g].nplanes = c->tc3_ok ? bp.group_nplanes[g] : 0;
     }
     c->tc_plane_beg = bp.plane_beg;
+    for (size_t g = 0; g < c->tri_groups.size(); ++g) {
+        c->tri_groups[g].boxes = c->tri_boxes + bp.tri_first[g];
+        c->tri_groups[g].nboxes = bp.tri_count[g];
+    }
+    c->tri_box_at = bp.tri_at;
+    c->n_xplanes = (int)bp.n_xpl;
+    c->xplane_beg = bp.xpl_beg;
     for (size_t g = 0; g < c->rx_groups.size(); ++g) {
         c->rx_groups[g].tiles = c->rx_tiles + bp.rx_group_first[g];
         c->rx_groups[g].ntiles = bp.rx_group_ntiles[g];
@@ -744,6 +781,22 @@ scola_status build(scola_ctx *c, const std::vector<BoxGeom> &all_geo) {
             c->tc_groups.push_back(G);
         }
     }
+    // FDA order 2: the x axis by elimination (k_dst_tri.cu)
+    if (p.fda_order == 2)
+        for (auto &kv : c->tbl_of) {
+            TriGroup G;
+            G.Ng = kv.first;
+            G.boxes = nullptr;
+            G.nboxes = 0;
+            G.mu_off = (long long)arena.size();
+            for (int l = 1; l <= G.Ng; ++l) {
+                const double s1 = std::sin(M_PI * l / (2.0 * (G.Ng + 1)));
+                arena.push_back((float)(4.0 * s1 * s1));
+            }
+            const double dg = dg_of_ng[G.Ng], sc = 2.0 / (G.Ng + 1);
+            G.kappa = (float)(-dg * dg * sc * sc);
+            c->tri_groups.push_back(G);
+        }
     double r = 0;
     for (const auto &g : all_geo) r += std::pow((double)g.nsc, 3);
     c->r = r / (double)c->N3;
@@ -817,7 +870,7 @@ scola_status build(scola_ctx *c, const std::vector<BoxGeom> &all_geo) {
     // every batch's layout (box descriptors kept; list lengths and arena sizes maxed)
     long long P = 0, M = 0, MP = 0, SH = 0, NK = 0, dep = 0;
     long long L_pch = 0, L_tch = 0, L_shch = 0, L_zit = 0, L_cit = 0, L_mch = 0, L_ppch = 0, L_sbr = 0, L_tct = 0,
-              L_pl = 0, L_rx = 0;
+              L_pl = 0, L_rx = 0, L_xp = 0;
     int max_count = 0;
     for (int k = 0; k < nbatch; ++k) {
         BatchPlan bp;
@@ -841,6 +894,7 @@ scola_status build(scola_ctx *c, const std::vector<BoxGeom> &all_geo) {
         L_tct = std::max(L_tct, bp.n_tct);
         L_pl = std::max(L_pl, bp.n_planes);
         L_rx = std::max(L_rx, bp.n_rxt);
+        L_xp = std::max(L_xp, bp.n_xpl);
         max_count = std::max(max_count, n);
         c->P_all += bp.P;
         for (const BoxGeom &g : bp.geo) c->M_all += (long long)g.ng * g.ng * g.ng;
@@ -862,6 +916,8 @@ scola_status build(scola_ctx *c, const std::vector<BoxGeom> &all_geo) {
     if (c->use_tc) CS(dev_alloc(&c->tc_tiles, L_tct));
     if (c->tc3_ok) CS(dev_alloc(&c->tc_planes, L_pl));
     if (c->rx_ok) CS(dev_alloc(&c->rx_tiles, L_rx));
+    CS(dev_alloc(&c->tri_boxes, max_count));
+    CS(dev_alloc(&c->xplanes, L_xp));
     c->cap_P = P;
     c->cap_M = M;
     c->cap_MP = MP;
@@ -887,6 +943,8 @@ scola_status build(scola_ctx *c, const std::vector<BoxGeom> &all_geo) {
 
     if ((!c->use_tc && !c->rx) || c->dst_auto) CK(init_pm_kernels(*c));     // the FP32 DST passes
     CK(init_deposit_kernels());
+    CK(init_tri_kernel());
+    CK(init_small_kernels());
     for (int i = 0; i < 4; ++i) CK(cudaEventCreate(&c->ev[i]));
     for (int i = 0; i < 2; ++i) CK(cudaEventCreate(&c->tc_ev[i]));
     CK(cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking));
@@ -904,43 +962,40 @@ scola_status build(scola_ctx *c, const std::vector<BoxGeom> &all_geo) {
 
 // A.1-A.2 on the full box into the context's grids.
 scola_status run_lpt(scola_ctx *c, const float *w, float *delta_out) {
-    const long long before = c->launches;
     const float invN3 = (float)(1.0 / (double)c->N3);
-    CF(cufftExecR2C(c->plan_r2c, const_cast<cufftReal *>(reinterpret_cast<const cufftReal *>(w)), c->ck));
+    CT(cufftExecR2C(c->plan_r2c, const_cast<cufftReal *>(reinterpret_cast<const cufftReal *>(w)), c->ck));
     CK(launch_colour(*c, c->ck));
     const size_t cbytes = sizeof(cufftComplex) * (size_t)c->Np * c->Np * (c->Np / 2 + 1);
     if (delta_out) {
         CK(cudaMemcpyAsync(c->ct, c->ck, cbytes, cudaMemcpyDeviceToDevice, c->stream));
-        CF(cufftExecC2R(c->plan_c2r, c->ct, delta_out));
+        CT(cufftExecC2R(c->plan_c2r, c->ct, delta_out));
     }
     CK(launch_inv_laplacian(*c, c->ck, c->cp, 1.0f));
     CK(cudaMemcpyAsync(c->ct, c->cp, cbytes, cudaMemcpyDeviceToDevice, c->stream));
-    CF(cufftExecC2R(c->plan_c2r, c->ct, c->phi1));
+    CT(cufftExecC2R(c->plan_c2r, c->ct, c->phi1));
     CK(launch_gradient(*c, c->phi1, c->psi1));
     if (c->prm.lpt_order == 1) {
         // Zel'dovich frame: no second-order potential or displacements
         CK(cudaMemsetAsync(c->phi2, 0, sizeof(float) * (size_t)c->N3, c->stream));
         CK(cudaMemsetAsync(c->psi2, 0, sizeof(float) * 3 * (size_t)c->N3, c->stream));
-        c->lpt_kernels = c->launches - before;
-        c->lpt_done = true;
+            c->lpt_done = true;
         return SCOLA_OK;
     }
     for (int a = 0; a < 3; ++a) {
         CK(launch_second_derivative(*c, c->cp, c->ct, a, a));
-        CF(cufftExecC2R(c->plan_c2r, c->ct, c->g[a]));
+        CT(cufftExecC2R(c->plan_c2r, c->ct, c->g[a]));
     }
     CK(launch_source_init(*c, c->g[0], c->g[1], c->g[2], c->g[3]));
     const int pairs[3][2] = {{0, 1}, {0, 2}, {1, 2}};
     for (auto &pr : pairs) {
         CK(launch_second_derivative(*c, c->cp, c->ct, pr[0], pr[1]));
-        CF(cufftExecC2R(c->plan_c2r, c->ct, c->g[0]));
+        CT(cufftExecC2R(c->plan_c2r, c->ct, c->g[0]));
         CK(launch_source_sub(*c, c->g[0], c->g[3]));
     }
-    CF(cufftExecR2C(c->plan_r2c, c->g[3], c->ct));
+    CT(cufftExecR2C(c->plan_r2c, c->g[3], c->ct));
     CK(launch_inv_laplacian(*c, c->ct, c->ct, invN3));
-    CF(cufftExecC2R(c->plan_c2r, c->ct, c->phi2));
+    CT(cufftExecC2R(c->plan_c2r, c->ct, c->phi2));
     CK(launch_gradient(*c, c->phi2, c->psi2));
-    c->lpt_kernels = c->launches - before;
     c->lpt_done = true;
     return SCOLA_OK;
 }
@@ -1482,7 +1537,7 @@ void scola_destroy(scola_ctx *c) {
         cufftDestroy(c->plan_c2r);
     }
     void *ptrs[] = {c->boxes, c->all_boxes, c->all_coef, c->all_coefL, c->coef, c->coefL, c->tables, c->table_arena, c->pchunks, c->tchunks, c->shchunks,
-                    c->zitems, c->citems, c->mchunks, c->ppchunks, c->tc_tiles, c->tc_planes, c->rx_tiles, c->dev_err, c->ckpt, c->ckpt_phi, c->seg, c->fin,
+                    c->zitems, c->citems, c->mchunks, c->ppchunks, c->tc_tiles, c->tc_planes, c->rx_tiles, c->tri_boxes, c->xplanes, c->dev_err, c->ckpt, c->ckpt_phi, c->seg, c->fin,
                     c->adj, c->lamG, c->lam_phi_pad, c->adj_in, c->adj_out, c->lam_shell, c->lamPsi1,
                     c->lamPsi2, c->lam_phi1, c->lam_phi2, c->d2, c->lam_d2, c->part, c->dep_acc, c->kcount,
                     c->koffs, c->kcursor, c->sentries, c->sbricks,
@@ -2005,7 +2060,7 @@ scola_status scola_selftest_wait_timeout(scola_ctx *c, double wait_seconds) {
     }
     CS(scola_device_status(c));                                // nothing pending before the test
     c->tc_stall_ns = (unsigned long long)(wait_seconds * 1e9);
-    const cudaError_t e = launch_poisson_tc_pass(*c, 0);       // work2 -> work: scratch meshes only
+    const cudaError_t e = launch_tc_selftest_pass(*c);         // work2 -> work: scratch meshes only
     c->tc_stall_ns = 0;
     CK(e);
     return scola_device_status(c);

@@ -71,6 +71,18 @@ struct TcGroup {                  // one tensor-core DST launch group: boxes sha
     long long lam_off;            // eigenvalues in table_arena
 };
 
+struct TriGroup {                 // the elimination along x (FDA order 2): boxes sharing Ng
+    int Ng;
+    Chunk *boxes;                 // device list of the bound batch's boxes
+    int nboxes;
+    long long mu_off;             // 4 sin^2 t_l in table_arena
+    float kappa;                  // -dg^2 (2 / (Ng + 1))^2
+};
+
+// The plane pass (k_dst_plane.cu): y and x forward, division, x and y inverse of a z-frequency
+// plane; z and y forward, or z and y inverse into the padded potential, of an x plane.
+enum PlaneMode { kPlaneSolve = 0, kPlaneForward = 1, kPlaneInverse = 2 };
+
 struct RxGroup {                  // one radix DST launch group: boxes sharing Ng
     int Ng, P, L, logL, R;        // DFT length P = Ng + 1, Bluestein length L, pencil pairs per tile
     Chunk *tiles;                 // device (box, tile of 2 R rows of the box)
@@ -158,6 +170,12 @@ struct Ctx {
     std::vector<RxGroup> rx_groups;
     Chunk *rx_tiles = nullptr;
     std::vector<int> rx_tile_beg, rx_tile_end;        // each box's tile range in rx_tiles
+    // FDA order 2: the boxes by Ng for the elimination along x, and every x plane of every box
+    std::vector<TriGroup> tri_groups;
+    Chunk *tri_boxes = nullptr;
+    std::vector<int> tri_box_at;                      // each box's place in tri_boxes
+    Chunk *xplanes = nullptr;  int n_xplanes = 0;     // (box, plane i): small meshes (k_dst_small.cu)
+    std::vector<int> xplane_beg;                      // each box's first plane
     int view_box = -1;                                // >= 0: launches restricted to this box
     int *dev_err = nullptr;                           // set by kernels whose bounded waits expired
     float *part = nullptr;
@@ -260,7 +278,12 @@ cudaError_t init_deposit_kernels();
 int tc_plan_stages(int Ng, int &Npad, int &nkc, bool zm = false);
 bool plane_supported(int Ng);    // the three-pass solve: Ng <= 96, Ng % 4 == 0
 cudaError_t init_plane_kernel();
-cudaError_t launch_plane_pass(Ctx &c, const std::vector<TcGroup> &groups, const float *in, float *out);
+cudaError_t launch_plane_pass(Ctx &c, const std::vector<TcGroup> &groups, PlaneMode mode, const float *in, float *out);
+cudaError_t init_tri_kernel();
+cudaError_t launch_tri_pass(Ctx &c, float *mesh);
+bool small_supported(const Ctx &c);
+cudaError_t init_small_kernels();
+cudaError_t launch_small_pass(Ctx &c, int pass, const float *in, float *w1, float *out_pad);
 // radix DST (k_dst_radix.cu): plan of one Ng, its host tables appended to the arena
 void rx_plan(int Ng, int &P, int &L, int &logL, int &R);
 bool rx_supported(int Ng);
@@ -272,7 +295,7 @@ bool tc_supported(int Ng);
 bool tc_folded(int Ng);          // Ng > 128: the mirror-symmetric half-size form
 bool tc_ragged(int Ng);          // rows not 16-byte pitched for TMA: plain loads and stores
 cudaError_t init_tc_kernels();
-cudaError_t launch_poisson_tc(Ctx &c);
+cudaError_t launch_tc_selftest_pass(Ctx &c);
 cudaError_t launch_poisson_tc_pass(Ctx &c, int pass);
 cudaError_t launch_poisson_tc_buffers(Ctx &c, const float *in, float *w1, float *w2,
                                       float *out_pad);

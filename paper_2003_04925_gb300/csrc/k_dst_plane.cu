@@ -1,14 +1,21 @@
-// Dirichlet Poisson solve in three mesh passes on the tensor cores: the plane pass
+// Dirichlet Poisson solve in three mesh passes on the tensor cores: the plane passes
 // (App. C, Eqs. 63-71).
 //
-// The solve of a box mesh with Ng <= 96 and Ng % 4 == 0 runs as
+// The solve of a box mesh with Ng <= 96 and Ng % 4 == 0 runs, at FDA order 2, as
+//   pass 1  kPlaneForward  every x plane i of src, held in shared memory, is transformed along z
+//                          and y                                        -> W1[i][m][n]
+//   pass 2  elimination along x (k_dst_tri.cu), in place
+//   pass 3  kPlaneInverse  every x plane of W1 is transformed back along z and y and written to
+//                          the padded potential
+// (two of the four transforms a plane, so each pass is bound by HBM more than by its chain of
+// products: 64 boxes of 96^3 take 107 + 106 + 123 us; the order 4/6 scheme below 99 + 185 + 111),
+// and at orders 4 and 6, where the Laplacian is not tridiagonal, as
 //   pass 1  z+     the one-axis pass of k_dst_tc.cu:   src[i][j][k] -> W1[n][i][j]
-//   pass 2  plane  this kernel: every z-frequency plane n of W1, held in shared memory, is
-//                  transformed along y and x, divided by lambda_l + lambda_m + lambda_n, and
-//                  transformed back along x and y                -> W2[n][i'][j']
+//   pass 2  kPlaneSolve    every z-frequency plane n of W1 is transformed along y and x, divided by
+//                          lambda_l + lambda_m + lambda_n, and transformed back along x and y
+//                                                                       -> W2[n][i'][j']
 //   pass 3  z-     the one-axis pass reading W2 plane by plane (k_dst_tc.cu, P_ZM), writing
-//                  the padded potential in its natural [i][j][k] layout
-// so the mesh crosses device memory three times per solve instead of six.
+//                  the padded potential in its natural [i][j][k] layout.
 //
 // Each step is D = S X^T with the sine matrix S (S_kn = sin(pi (k+1)(n+1)/(Ng+1))) as the
 // M = 128 operand and the plane's Ng rows as the N operand, both split into FP16 hi and lo
@@ -30,8 +37,15 @@
 //   step 2  rows m,   K = i   ->  lanes l  (x frequency), columns m   (then / lambda sum)
 //   step 3  rows l,   K = m   ->  lanes j' (y),           columns l
 //   step 4  rows j',  K = l   ->  lanes i' (x),           columns j'  -> row i' of W2[n]
+// (kPlaneForward: rows j, K = k -> lanes n; rows n, K = j -> lanes m: row m of W1[i].
+// kPlaneInverse: rows m, K = n -> lanes k'; rows k', K = m -> lanes j': row j' of the potential.)
+// The cross products are issued before the hi x hi ones of a step: every MMA rounds its running
+// sum, and this order leaves Ng / 16 roundings at full magnitude instead of 3 Ng / 16 (a force
+// evaluation on 64 boxes of 96^3: error against FP64 8e-6 -> 3e-6).
 // The output plane is written row by row into the group's operand buffer (free once the
-// step-4 MMAs are complete; the staging layout) and leaves by tensor store.
+// last step's MMAs are complete; the staging layout) and leaves by tensor store, or for the
+// padded potential, whose rows have no tensor map common to all boxes, by the group's own
+// 16-byte stores (a warp set apart for them held the groups up: 152 us against 123 us).
 // Three planes are in flight per CTA (three operand buffers, three accumulators): while
 // the epilogues turn two planes' accumulators into their next operands, the tensor cores
 // run the third plane's step.  The FP32 planes land in two staging buffers by tensor copy;
@@ -87,6 +101,7 @@ struct PlaneArgs {
     PlaneGroupArgs grp[kPlGroups];
     int ngroups;
     const BoxDesc *boxes;
+    float *out;                  // kPlaneInverse: the padded potential
     int *err;
     int lo_lo;
 };
@@ -148,7 +163,9 @@ __device__ __forceinline__ float row_max(const float (&x)[kPlMaxN / 16][16]) {
     return m[0];
 }
 
+template <int MODE>
 __global__ void __launch_bounds__(kPlThreads, 1) k_dst_plane(const __grid_constant__ PlaneArgs A) {
+    constexpr int STEPS = MODE == kPlaneSolve ? 4 : 2;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char *base = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
     int gi = 0;
@@ -197,7 +214,7 @@ __global__ void __launch_bounds__(kPlThreads, 1) k_dst_plane(const __grid_consta
             mbar_init(&opready[e], kPlRows);
             mbar_init(&accfull[e], 1);
             mbar_init(&outw[e], kPlRows);
-            mbar_init(&outfree[e], 1);
+            mbar_init(&outfree[e], MODE == kPlaneInverse ? kPlRows : 1);
         }
         mbar_init(drain, 1);
         *abort_flag = 0;
@@ -282,7 +299,7 @@ __global__ void __launch_bounds__(kPlThreads, 1) k_dst_plane(const __grid_consta
             const bool lo_lo = A.lo_lo != 0;
             bool ok = true;
             for (long long q = 0; q < ntrip && ok && !*abort_flag; ++q)
-                for (int s = 1; s <= 4 && ok; ++s)
+                for (int s = 1; s <= STEPS && ok; ++s)
                     for (int e = 0; e < kPlBuf; ++e) {
                         if (q * kPlBuf + e >= my_items) break;
                         if (!mbar_spin(&opready[e], (uint32_t)((s - 1) & 1), abort_flag)) {
@@ -296,13 +313,19 @@ __global__ void __launch_bounds__(kPlThreads, 1) k_dst_plane(const __grid_consta
                         // FP16 columns is 32 bytes of the swizzled row, 8 TMEM columns of S
                         const uint64_t bh0 = sw128_desc(smem_u32(ops + (size_t)e * 2 * bhalf));
                         const uint64_t bl0 = bh0 + (bhalf >> 4);
+                        // the small cross products first: every MMA rounds its sum to the
+                        // accumulator's precision, and while that holds the lo terms alone it
+                        // rounds at their level (a third of the roundings at full magnitude)
                         for (int t = 0; t < nk16; ++t) {
                             const uint64_t off = (uint64_t)(t >> 2) * (och >> 4) + (uint64_t)((t & 3) * 2);
                             const uint32_t ah = tmem + (uint32_t)(t * 8), al = ah + (uint32_t)kSCols;
-                            mma_f16_ts(d, ah, bh0 + off, idesc, t ? 1u : 0u);
-                            mma_f16_ts(d, ah, bl0 + off, idesc, 1);
+                            if (lo_lo) mma_f16_ts(d, al, bl0 + off, idesc, t ? 1u : 0u);
+                            mma_f16_ts(d, ah, bl0 + off, idesc, t || lo_lo ? 1u : 0u);
                             mma_f16_ts(d, al, bh0 + off, idesc, 1);
-                            if (lo_lo) mma_f16_ts(d, al, bl0 + off, idesc, 1);
+                        }
+                        for (int t = 0; t < nk16; ++t) {
+                            const uint64_t off = (uint64_t)(t >> 2) * (och >> 4) + (uint64_t)((t & 3) * 2);
+                            mma_f16_ts(d, tmem + (uint32_t)(t * 8), bh0 + off, idesc, 1);
                         }
                         mma_commit(&accfull[e]);
                     }
@@ -356,7 +379,7 @@ __global__ void __launch_bounds__(kPlThreads, 1) k_dst_plane(const __grid_consta
                 // the operand buffer holds the previous plane's output until its tensor store
                 // has read it (issued by the group's thread 0, which signals here)
                 if (q > 0) {
-                    if (row == 0) {
+                    if (MODE != kPlaneInverse && row == 0) {
                         bulk_wait_read();
                         mbar_arrive(&outfree[e]);
                     }
@@ -372,7 +395,7 @@ __global__ void __launch_bounds__(kPlThreads, 1) k_dst_plane(const __grid_consta
             fence_proxy_async();
             mbar_arrive(&opready[e]);
             const float lam_row = row < Ng ? lam[row] : 0.0f, lam_n = lam[n];
-            for (int s = 1; s <= 4; ++s) {
+            for (int s = 1; s <= STEPS; ++s) {
                 if (!mbar_wait(&accfull[e], (uint32_t)((s - 1) & 1), abort_flag)) {
                     ok = false;
                     break;
@@ -403,7 +426,7 @@ __global__ void __launch_bounds__(kPlThreads, 1) k_dst_plane(const __grid_consta
                         const float4 u4 = u_in[4 * c + jq];
                         const float uu[4] = {u4.x, u4.y, u4.z, u4.w};
                         float ll[4] = {0.f, 0.f, 0.f, 0.f};
-                        if (s == 2) {
+                        if (STEPS == 4 && s == 2) {
                             const float4 l4 = lam4[4 * c + jq];
                             ll[0] = l4.x, ll[1] = l4.y, ll[2] = l4.z, ll[3] = l4.w;
                         }
@@ -411,11 +434,11 @@ __global__ void __launch_bounds__(kPlThreads, 1) k_dst_plane(const __grid_consta
                         for (int t = 0; t < 4; ++t) {
                             const int j = 4 * jq + t;
                             float y = x[c][j] * uu[t];
-                            if (s == 2) y = __fdividef(y, lam_row + ll[t] + lam_n);
+                            if (STEPS == 4 && s == 2) y = __fdividef(y, lam_row + ll[t] + lam_n);
                             x[c][j] = y;
                         }
                     }
-                if (s == 4) {
+                if (s == STEPS) {
                     // row i' of the output plane into the operand buffer (32-column chunks,
                     // 128-byte swizzle, as the copies bring the planes in); thread 0 of the
                     // group stores the plane once every row is written
@@ -434,7 +457,7 @@ __global__ void __launch_bounds__(kPlThreads, 1) k_dst_plane(const __grid_consta
                     fence_proxy_async();
                     tc_fence_before();
                     mbar_arrive(&outw[e]);
-                    if (row == 0) {
+                    if (MODE != kPlaneInverse && row == 0) {
                         if (!mbar_wait(&outw[e], (uint32_t)(q & 1), abort_flag)) {
                             ok = false;
                             break;
@@ -442,6 +465,31 @@ __global__ void __launch_bounds__(kPlThreads, 1) k_dst_plane(const __grid_consta
                         const int y = (int)(m_off / Ng + (long long)n * Ng);     // row (n, i' = 0)
                         for (int c = 0; c < nka; ++c) tma_store_2d(&G.out_map, c * 32, y, smem_u32(hi + (size_t)c * och));
                         bulk_commit();
+                    }
+                    if (MODE == kPlaneInverse) {
+                        // the padded potential's rows start on a 16-byte grid that differs from
+                        // box to box (no common tensor map): once every row is written, the
+                        // group copies the plane out, 16 bytes a lane along the rows
+                        if (!mbar_wait(&outw[e], (uint32_t)(q & 1), abort_flag)) {
+                            ok = false;
+                            break;
+                        }
+                        const int gp = A.boxes[it.box].gpad, S = Ng + 2 * gp, r4 = Ng / 4;
+                        float *dst = A.out + A.boxes[it.box].pp_off + (((n + gp) * S + gp) * S + gp);
+                        int r = row / r4, u = row - r * r4;                 // row, 16-byte unit
+                        const int dr = kPlRows / r4, du = kPlRows - dr * r4;
+#pragma unroll 4
+                        for (int f = row; f < Ng * r4; f += kPlRows) {
+                            *reinterpret_cast<float4 *>(dst + r * S + 4 * u) = *reinterpret_cast<const float4 *>(
+                                hi + (uint32_t)(u >> 3) * och + sw128_offset(r, 4 * (u & 7)));
+                            r += dr;
+                            u += du;
+                            if (u >= r4) {
+                                u -= r4;
+                                ++r;
+                            }
+                        }
+                        mbar_arrive(&outfree[e]);
                     }
                 } else {
                     const int sr = row_exp(row_max(x));
@@ -454,7 +502,7 @@ __global__ void __launch_bounds__(kPlThreads, 1) k_dst_plane(const __grid_consta
             }
         }
         // thread 0's tensor stores complete before the CTA exits
-        if (row == 0) bulk_wait_all();
+        if (MODE != kPlaneInverse && row == 0) bulk_wait_all();
         if (!ok) *abort_flag = 1;
     }
 
@@ -516,13 +564,18 @@ bool plane_supported(int Ng) {
 }
 
 cudaError_t init_plane_kernel() {
-    return cudaFuncSetAttribute(k_dst_plane, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPlSmemBudget);
+    for (const void *f : {(const void *)k_dst_plane<kPlaneSolve>, (const void *)k_dst_plane<kPlaneForward>,
+                          (const void *)k_dst_plane<kPlaneInverse>}) {
+        const cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPlSmemBudget);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 // The plane pass over the given Ng groups (at most kPlGroups per launch): items are (box,
 // plane) pairs of every box of each group; the persistent grid is split among the groups in
 // proportion to their work (planes x Ng^2).
-cudaError_t launch_plane_pass(Ctx &c, const std::vector<TcGroup> &groups, const float *in, float *out) {
+cudaError_t launch_plane_pass(Ctx &c, const std::vector<TcGroup> &groups, PlaneMode mode, const float *in, float *out) {
     for (size_t g0 = 0; g0 < groups.size(); g0 += kPlGroups) {
         const int ng = (int)std::min(groups.size() - g0, (size_t)kPlGroups);
         PlaneArgs a;
@@ -543,7 +596,7 @@ cudaError_t launch_plane_pass(Ctx &c, const std::vector<TcGroup> &groups, const 
             P.Npad = (G.Ng + 15) / 16 * 16;
             P.nka = G.nkc;
             cudaError_t e = plane_map(c, in, P.Ng, P.Npad, &P.in_map);
-            if (e == cudaSuccess) e = plane_map(c, out, P.Ng, P.Ng, &P.out_map);
+            if (e == cudaSuccess && mode != kPlaneInverse) e = plane_map(c, out, P.Ng, P.Ng, &P.out_map);
             if (e != cudaSuccess) return e;
             P.items = G.planes;
             P.nitems = G.nplanes;
@@ -559,9 +612,12 @@ cudaError_t launch_plane_pass(Ctx &c, const std::vector<TcGroup> &groups, const 
         }
         a.ngroups = ng;
         a.boxes = c.boxes;
+        a.out = out;
         a.err = c.dev_err;
         a.lo_lo = c.tc_lo_lo ? 1 : 0;
-        k_dst_plane<<<cta0, kPlThreads, smem, c.stream>>>(a);
+        if (mode == kPlaneForward) k_dst_plane<kPlaneForward><<<cta0, kPlThreads, smem, c.stream>>>(a);
+        else if (mode == kPlaneInverse) k_dst_plane<kPlaneInverse><<<cta0, kPlThreads, smem, c.stream>>>(a);
+        else k_dst_plane<kPlaneSolve><<<cta0, kPlThreads, smem, c.stream>>>(a);
         ++c.launches;
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;

@@ -88,7 +88,14 @@ constexpr int kTmemCols = 2 * kTN;   // double-buffered accumulator
 // Per epilogue warp: a 32 x 33 float block for transposing 32 columns x 32 rows.
 constexpr int kXposeBytes = 32 * 33 * 4;
 
-enum TcPass { P_F = 1, P_XF = 2, P_ZI = 3, P_YI = 4, P_XI = 5, P_ZM = 6 };   // P_F: z+ and y+
+enum TcPass { P_F = 1, P_XF = 2, P_ZI = 3, P_YI = 4, P_XI = 5, P_ZM = 6, P_M = 7, P_MI = 8 };   // P_F: z+ and y+
+// P_M, P_MI: the passes of the order-2 solve with the x axis by elimination (k_dst_tri.cu).  The
+// output index takes the middle place, out[hi][col][lo] for row (hi, lo), so that z+, y+, z-, y-
+// stay within each x plane and the mesh keeps x slowest:
+//   z+  src[i][j][k]  (i,j)  k    W[i][n][j]
+//   y+  W[i][n][j]    (i,n)  j    W[i][m][n]        (then the elimination along i)
+//   z-  W[i][m][n]    (i,m)  n    W[i][k'][m]
+//   y-  W[i][k'][m]   (i,k') m    Phi[i+2][j'+2][k'+2]   (P_MI; the scale is in the elimination)
 // P_ZM: the z inverse of the three-pass solve (k_dst_plane.cu), reading W2[n][i][j] plane by
 // plane: a tile is 256 consecutive cells q = (i, j) of the planes, its K chunk 16 planes n;
 // the tensor copy brings the [16 n][256 q] box unswizzled, the converters transpose it into
@@ -557,13 +564,17 @@ __global__ void __launch_bounds__(kThreads, 1) k_dst_tc(const __grid_constant__ 
                     if (row < (int)Ng2) {
                         const int rhi = row / Ng, rlo = row - rhi * Ng, gp = ti.pad, S = Ng + 2 * gp;
                         const float lhi = lam[rhi], llo = lam[rlo];
-                        float *dst = PASS == P_XI ? A.out + ti.pp_off + ((rhi + gp) * S + (rlo + gp)) : A.out + ti.m_off + row;
+                        float *dst = A.out + ti.m_off + row;
+                        long long step = Ng2;                        // between output columns
+                        if (PASS == P_XI) dst = A.out + ti.pp_off + ((gp * S + rhi + gp) * S + (rlo + gp)), step = S * S;
+                        if (PASS == P_M) dst = A.out + ti.m_off + ((long long)rhi * Ng2 + rlo), step = Ng;
+                        if (PASS == P_MI) dst = A.out + ti.pp_off + (((rhi + gp) * S + gp) * S + (rlo + gp)), step = S;
                         for (int nl = 0; nl < ncol; ++nl) {
                             const int nout = FOLD ? 2 * (n0 + nl) + parity : n0 + nl;
                             float y = buf[nl * 32 + ((((lane >> 2) ^ nl) & 7) << 2) + (lane & 3)];
                             if (PASS == P_XF) y = __fdividef(y, lam[nout] + lhi + llo);
-                            if (PASS == P_XI) dst[(long long)(nout + gp) * S * S] = y * scale;
-                            else dst[(long long)nout * Ng2] = y;
+                            if (PASS == P_XI) y *= scale;
+                            dst[nout * step] = y;
                         }
                     }
                 } else if (R < Ng2) {
@@ -585,6 +596,12 @@ __global__ void __launch_bounds__(kThreads, 1) k_dst_tc(const __grid_constant__ 
                             const long long S = Ng + 2 * G;
                             float *p = A.out + ti.pp_off + ((long long)(nout + G) * S + (rhi + G)) * S + (rlo + G);
                             *reinterpret_cast<float4 *>(p) = make_float4(x.x * scale, x.y * scale, x.z * scale, x.w * scale);
+                        } else if (PASS == P_MI) {
+                            const int G = ti.pad, S = Ng + 2 * G;
+                            *reinterpret_cast<float4 *>(A.out + ti.pp_off +
+                                                        (((rhi + G) * S + (nout + G)) * S + (rlo + G))) = x;
+                        } else if (PASS == P_M) {
+                            *reinterpret_cast<float4 *>(A.out + ti.m_off + ((rhi * Ng + nout) * Ng + rlo)) = x;
                         } else {
                             if (PASS == P_XF) {
                                 const float ln = lam[nout];
@@ -784,6 +801,8 @@ cudaError_t init_tc_kernels() {
     if ((e = set_tc_attr<P_ZI>())) return e;
     if ((e = set_tc_attr<P_YI>())) return e;
     if ((e = set_tc_attr<P_ZM>())) return e;
+    if ((e = set_tc_attr<P_M>())) return e;
+    if ((e = set_tc_attr<P_MI>())) return e;
     if ((e = init_plane_kernel())) return e;
     return set_tc_attr<P_XI>();
 }
@@ -830,63 +849,76 @@ std::vector<std::vector<TcGroup>> tc_launches(const Ctx &c) {
     return out;
 }
 
-cudaError_t launch_poisson_tc_pass(Ctx &c, int pass) {
-    if (c.tc3) {
-        // three passes: source (work2) -> work (z+) -> work2 (plane) -> phi (z-)
-        if (pass >= 3) return cudaSuccess;
-        cudaError_t e = cudaSuccess;
-        for (const auto &L : tc_launches(c)) {
-            if (pass == 0) e = run_tc_pass<P_F>(c, L, c.work2, c.work);
-            else if (pass == 1) e = launch_plane_pass(c, L, c.work, c.work2);
-            else e = run_tc_pass<P_ZM>(c, L, c.work2, c.phi);
-            if (e != cudaSuccess) return e;
-        }
-        return cudaSuccess;
-    }
-    // buffers: source (work2) -> work -> work2 -> work -> work2 -> work -> phi
-    cudaError_t e = cudaSuccess;
-    for (const auto &L : tc_launches(c)) {
+// Pass `pass` of the solve in -> w1, w2 -> out_pad.  FDA order 2 takes the x axis by elimination:
+//   three passes (c.tc3)  plane (z, y forward)  elimination  plane (z, y inverse)
+//   otherwise             z+  y+  elimination  z-  y-
+// Orders 4 and 6 (no tridiagonal form) divide in sine space:
+//   three passes          z+  plane (y, x, division, x, y)  z-
+//   otherwise             z+  y+  x+ with the division  z-  y-  x-
+// Passes beyond a form's last are empty.
+static cudaError_t tc_pass(Ctx &c, const std::vector<TcGroup> &L, int pass, const float *in, float *w1, float *w2,
+                           float *out_pad) {
+    const bool tri = c.prm.fda_order == 2;
+    if (c.tc3 && tri) {
         switch (pass) {
-            case 0: e = run_tc_pass<P_F>(c, L, c.work2, c.work); break;
-            case 1: e = run_tc_pass<P_F>(c, L, c.work, c.work2); break;
-            case 2: e = run_tc_pass<P_XF>(c, L, c.work2, c.work); break;
-            case 3: e = run_tc_pass<P_ZI>(c, L, c.work, c.work2); break;
-            case 4: e = run_tc_pass<P_YI>(c, L, c.work2, c.work); break;
-            case 5: e = run_tc_pass<P_XI>(c, L, c.work, c.phi); break;
-            default: return cudaErrorInvalidValue;
+            case 0: return launch_plane_pass(c, L, kPlaneForward, in, w1);
+            case 2: return launch_plane_pass(c, L, kPlaneInverse, w1, out_pad);
+            default: return cudaSuccess;
         }
+    }
+    if (c.tc3) {
+        switch (pass) {
+            case 0: return run_tc_pass<P_F>(c, L, in, w1);
+            case 1: return launch_plane_pass(c, L, kPlaneSolve, w1, w2);
+            case 2: return run_tc_pass<P_ZM>(c, L, w2, out_pad);
+            default: return cudaSuccess;
+        }
+    }
+    if (tri) {
+        switch (pass) {
+            case 0: return run_tc_pass<P_M>(c, L, in, w1);
+            case 1: return run_tc_pass<P_M>(c, L, w1, w2);
+            case 3: return run_tc_pass<P_M>(c, L, w2, w1);
+            case 4: return run_tc_pass<P_MI>(c, L, w1, out_pad);
+            default: return cudaSuccess;
+        }
+    }
+    switch (pass) {
+        case 0: return run_tc_pass<P_F>(c, L, in, w1);
+        case 1: return run_tc_pass<P_F>(c, L, w1, w2);
+        case 2: return run_tc_pass<P_XF>(c, L, w2, w1);
+        case 3: return run_tc_pass<P_ZI>(c, L, w1, w2);
+        case 4: return run_tc_pass<P_YI>(c, L, w2, w1);
+        case 5: return run_tc_pass<P_XI>(c, L, w1, out_pad);
+        default: return cudaErrorInvalidValue;
+    }
+}
+
+// A pass over every box of the view: the launches of each Ng form in turn (the elimination
+// groups the boxes itself).
+static cudaError_t tc_pass_all(Ctx &c, int pass, const float *in, float *w1, float *w2, float *out_pad) {
+    if (c.prm.fda_order == 2 && pass == (c.tc3 ? 1 : 2)) return launch_tri_pass(c, c.tc3 ? w1 : w2);
+    for (const auto &L : tc_launches(c)) {
+        const cudaError_t e = tc_pass(c, L, pass, in, w1, w2, out_pad);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
 }
 
-cudaError_t launch_poisson_tc(Ctx &c) {
-    for (int p = 0; p < 6; ++p) {
-        cudaError_t e = launch_poisson_tc_pass(c, p);
-        if (e != cudaSuccess) return e;
-    }
-    return cudaSuccess;
-}
-// (launch_poisson in k_pm.cu uses the same sequence through launch_poisson_buffers.)
+cudaError_t launch_poisson_tc_pass(Ctx &c, int pass) { return tc_pass_all(c, pass, c.work2, c.work, c.work2, c.phi); }
 
 cudaError_t launch_poisson_tc_buffers(Ctx &c, const float *in, float *w1, float *w2, float *out_pad) {
-    cudaError_t e = cudaSuccess;
-    if (c.tc3) {
-        for (const auto &L : tc_launches(c)) {
-            e = run_tc_pass<P_F>(c, L, in, w1);
-            if (e == cudaSuccess) e = launch_plane_pass(c, L, w1, w2);
-            if (e == cudaSuccess) e = run_tc_pass<P_ZM>(c, L, w2, out_pad);
-            if (e != cudaSuccess) return e;
-        }
-        return cudaSuccess;
+    for (int pass = 0; pass < 6; ++pass) {
+        const cudaError_t e = tc_pass_all(c, pass, in, w1, w2, out_pad);
+        if (e != cudaSuccess) return e;
     }
+    return cudaSuccess;
+}
+
+// One z+ pass work2 -> work (scratch meshes) for the failure-detection self-test.
+cudaError_t launch_tc_selftest_pass(Ctx &c) {
     for (const auto &L : tc_launches(c)) {
-        e = run_tc_pass<P_F>(c, L, in, w1);
-        if (e == cudaSuccess) e = run_tc_pass<P_F>(c, L, w1, w2);
-        if (e == cudaSuccess) e = run_tc_pass<P_XF>(c, L, w2, w1);
-        if (e == cudaSuccess) e = run_tc_pass<P_ZI>(c, L, w1, w2);
-        if (e == cudaSuccess) e = run_tc_pass<P_YI>(c, L, w2, w1);
-        if (e == cudaSuccess) e = run_tc_pass<P_XI>(c, L, w1, out_pad);
+        const cudaError_t e = run_tc_pass<P_F>(c, L, c.work2, c.work);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;

@@ -433,6 +433,13 @@ cudaError_t init_pm_kernels(Ctx &c) {
 cudaError_t launch_poisson_buffers(Ctx &c, const float *in, float *w1, float *w2, float *out_pad) {
     if (c.rx) return launch_poisson_rx_buffers(c, in, w1, w2, out_pad);
     if (c.use_tc) return launch_poisson_tc_buffers(c, in, w1, w2, out_pad);
+    if (small_supported(c)) {
+        for (int pass = 0; pass < 3; ++pass) {
+            const cudaError_t e = launch_small_pass(c, pass, in, w1, out_pad);
+            if (e != cudaSuccess) return e;
+        }
+        return cudaSuccess;
+    }
     switch (c.max_R) {
         case 1: return poisson_R<1>(c, in, w1, w2, out_pad);
         case 2: return poisson_R<2>(c, in, w1, w2, out_pad);
@@ -453,6 +460,7 @@ cudaError_t launch_poisson_pass(Ctx &c, int pass) {
     // form has five passes, the tensor-core and radix forms six
     if (c.rx) return launch_poisson_rx_pass(c, pass);
     if (c.use_tc) return launch_poisson_tc_pass(c, pass);
+    if (small_supported(c)) return launch_small_pass(c, pass, c.work2, c.work, c.phi);
     if (pass == 5) return cudaSuccess;
     switch (c.max_R * 8 + pass) {
 #define SCOLA_PASS_CASES(R)                                                                     \
