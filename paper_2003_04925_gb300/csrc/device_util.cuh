@@ -192,11 +192,8 @@ __device__ __forceinline__ void shell_stencil(const BoxDesc &B, const int pc[3],
     }
 }
 
-// The same stencil with the offsets in FP64, for the FP64 accumulation of the C.3 shell: the
-// exact integer r times the box's FP64 reciprocal of den (two FP64 roundings, far below the
-// FP32 rounding of the result; FP64 division is slow on this GPU).
-__device__ __forceinline__ void shell_stencil_d(const BoxDesc &B, const int pc[3], int Ntile, int i0[3],
-                                                double f[3]) {
+// The same stencil with each offset as the exact remainder r of r / (2 Ng).
+__device__ __forceinline__ void shell_stencil_r(const BoxDesc &B, const int pc[3], int Ntile, int i0[3], int rem[3]) {
     const int t[3] = {B.tx, B.ty, B.tz};
     const int den = 2 * B.Ng;
 #pragma unroll
@@ -208,8 +205,32 @@ __device__ __forceinline__ void shell_stencil_d(const BoxDesc &B, const int pc[3
             --q;
         }
         i0[a] = t[a] * Ntile - B.Nbuf + q;
-        f[a] = (double)r * B.inv_2ng_d;
+        rem[a] = r;
     }
+}
+
+// Unevaluated sums h + l of two floats (about 47 significant bits), for the C.3 shell: FP64 runs
+// at 1/64 of the FP32 rate on this GPU.  Sums by Knuth's two-sum, products by one FMA remainder
+// (Dekker 1971, Knuth TAOCP vol. 2, 4.2.2); the _rn intrinsics keep the compiler from fusing.
+struct FloatPair {
+    float h, l;
+};
+
+__device__ __forceinline__ FloatPair two_sum(float a, float b) {
+    const float s = __fadd_rn(a, b), t = __fsub_rn(s, a);
+    return {s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t))};
+}
+
+// a + f (b - a)
+__device__ __forceinline__ FloatPair pair_lerp(FloatPair a, FloatPair b, FloatPair f) {
+    FloatPair d = two_sum(b.h, -a.h);
+    d.l = __fadd_rn(d.l, __fsub_rn(b.l, a.l));
+    const float th = __fmul_rn(f.h, d.h);
+    const float tl = __fmaf_rn(f.l, d.h, __fmaf_rn(f.h, d.l, __fmaf_rn(f.h, d.h, -th)));
+    FloatPair r = two_sum(a.h, th);
+    r.l = __fadd_rn(r.l, __fadd_rn(a.l, tl));
+    const float h = __fadd_rn(r.h, r.l);
+    return {h, __fsub_rn(r.l, __fsub_rn(h, r.h))};
 }
 
 __device__ __forceinline__ int wrap(int v, int n) {
