@@ -1731,7 +1731,7 @@ scola_status scola_set_checkpointing(scola_ctx *c, int32_t enable) {
     if (on) CS(alloc_checkpoints(c));
     if (on && !c->adj) {
         const long long P = c->cap_P, N3 = c->N3;
-        CS(dev_alloc(&c->adj, 15 * P));
+        CS(dev_alloc(&c->adj, 12 * P));
         CS(dev_alloc(&c->lamG, 4 * c->cap_MP));       // interleaved (x, y, z, unused) per padded cell
         CS(dev_alloc(&c->lam_phi_pad, c->cap_MP));
         CS(dev_alloc(&c->adj_in, c->cap_M));
@@ -1810,7 +1810,7 @@ scola_status backward_clear_global(scola_ctx *c) {
 // Clears the bound batch's backward state; the caller then sets its tile particles' state.
 scola_status backward_clear_batch(scola_ctx *c) {
     const size_t fb = sizeof(float);
-    CK(cudaMemsetAsync(c->adj, 0, fb * 15 * c->P, c->stream));
+    CK(cudaMemsetAsync(c->adj, 0, fb * 12 * c->P, c->stream));
     CK(cudaMemsetAsync(c->lam_shell, 0, fb * c->SH, c->stream));
     return SCOLA_OK;
 }
@@ -1822,16 +1822,15 @@ scola_status backward_clear_batch(scola_ctx *c) {
 // evaluation k from the coefficient table (k is passed on); otherwise the uniform scalars.
 scola_status reverse_step(scola_ctx *c, int k, const float *sk) {
     const long long P = c->P;
-    CK(launch_adj_kick_drift(*c, c->adj, kick_drift_coefficients(c->tt, k), k));
+    const float *phi = c->phi;
     if (c->ckpt_phi && c->ckpt_every == 1) {       // the potential the forward run kept
-        CK(cudaMemcpyAsync(c->phi, c->ckpt_phi + (size_t)k * c->MP, sizeof(float) * (size_t)c->MP,
-                           cudaMemcpyDeviceToDevice, c->stream));
+        phi = c->ckpt_phi + (size_t)k * c->MP;
     } else {
         CK(launch_deposit(*c, sk, P, (float)(1.0 / c->tt.D1[k]), nullptr, false, k));
         CK(launch_poisson(*c));
     }
     CK(cudaMemsetAsync(c->lamG, 0, sizeof(float) * 4 * c->MP, c->stream));
-    CK(launch_adj_interp(*c, sk, c->adj, c->lamG, (float)c->tt.D1[k], k));
+    CK(launch_adj_step(*c, sk, c->adj, kick_drift_coefficients(c->tt, k), phi, c->lamG, (float)c->tt.D1[k], k));
     CK(launch_adj_div(*c, c->lamG, c->lam_phi_pad, c->adj_in));
     CK(launch_poisson_buffers(*c, c->adj_in, c->work, c->work2, c->adj_out));
     CK(launch_adj_shell(*c, c->lam_phi_pad, c->adj_out, (float)c->tt.D1[k], c->lam_shell, k));

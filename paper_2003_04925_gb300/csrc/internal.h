@@ -233,7 +233,7 @@ struct Ctx {
     float *ckpt_phi = nullptr;
     float *seg = nullptr, *fin = nullptr;
     long long cap_P = 0, cap_M = 0, cap_MP = 0, cap_SH = 0;   // the largest batch's arena sizes
-    float *adj = nullptr;                             // 15 x P backward particle state
+    float *adj = nullptr;                             // 12 x P backward particle state
     float *lamG = nullptr, *lam_phi_pad = nullptr, *adj_in = nullptr, *adj_out = nullptr;
     float *lam_shell = nullptr, *lamPsi1 = nullptr, *lamPsi2 = nullptr;
     float *lam_phi1 = nullptr, *lam_phi2 = nullptr, *d2 = nullptr, *lam_d2 = nullptr;
@@ -344,8 +344,8 @@ cudaError_t launch_adj_final_xp(Ctx &c, const float *lam_x, const float *lam_p, 
 // the periodic CIC adjoint of the final density over the global positions
 cudaError_t launch_density_vjp(Ctx &c, const float *x, const float *lam_delta, float *lam_x);
 // k >= 0 with per-tile final scale factors: each box's factors of evaluation k (coef table)
-cudaError_t launch_adj_kick_drift(Ctx &c, float *adj, const KickDrift &kd, int k = -1);
-cudaError_t launch_adj_interp(Ctx &c, const float *s, float *adj, float *lamG, float D1, int k = -1);
+cudaError_t launch_adj_step(Ctx &c, const float *s, float *adj, const KickDrift &kd, const float *phi, float *lamG,
+                            float D1, int k = -1);
 cudaError_t launch_adj_div(Ctx &c, const float *lamG, float *lam_phi_pad, float *interior_out);
 cudaError_t launch_adj_shell(Ctx &c, const float *lam_phi_pad, const float *lam_src_pad, float D1,
                              float *lam_shell, int k = -1);
