@@ -215,10 +215,10 @@ void add_chunks(std::vector<Chunk> &v, int box, long long n, int per) {
 struct BatchPlan {
     std::vector<BoxGeom> geo;                          // the batch's boxes (its shape)
     std::vector<BoxDesc> boxes;
-    std::vector<Chunk> pch, tch, shch, zit, cit, mch, ppch, sbr, tct;
-    long long n_pch = 0, n_tch = 0, n_shch = 0, n_zit = 0, n_cit = 0, n_mch = 0, n_ppch = 0, n_sbr = 0,
+    std::vector<Chunk> pch, bch, tch, shch, zit, cit, mch, ppch, sbr, tct;
+    long long n_pch = 0, n_bch = 0, n_tch = 0, n_shch = 0, n_zit = 0, n_cit = 0, n_mch = 0, n_ppch = 0, n_sbr = 0,
               n_tct = 0;
-    std::vector<int> pbeg, shbeg, zbeg, cbeg, mbeg, sbbeg, tile_beg, tile_end, dep_groups;
+    std::vector<int> pbeg, bbeg, shbeg, zbeg, cbeg, mbeg, sbbeg, tile_beg, tile_end, dep_groups;
     std::vector<long long> group_first;                // per tensor-core group: first tile, count
     std::vector<int> group_ntiles;
     std::vector<Chunk> planes;                         // three-pass solve: (box, plane) per group
@@ -256,6 +256,7 @@ void plan_batch(const scola_ctx *c, const std::vector<BoxGeom> &tiling_geo, int 
     long long P = 0, M = 0, MP = 0, SH = 0, NK = 0;
     for (int b = 0; b < count; ++b) {
         bp.pbeg.push_back((int)bp.n_pch);
+        bp.bbeg.push_back((int)bp.n_bch);
         bp.shbeg.push_back((int)bp.n_shch);
         bp.zbeg.push_back((int)bp.n_zit);
         bp.cbeg.push_back((int)bp.n_cit);
@@ -285,7 +286,7 @@ void plan_batch(const scola_ctx *c, const std::vector<BoxGeom> &tiling_geo, int 
         B.p_off = P;
         B.m_off = M;
         // padded boxes (G = FDA order ghost layers per side) start G mod 4 floats past a
-        // 64-float boundary: with Ng % 4 == 0 the interior cells of every padded row
+        // 128-float boundary (a texture's base alignment): with Ng % 4 == 0 the interior cells of every padded row
         // (index G .. Ng + G - 1) then start 16-byte aligned
         const int G = p.fda_order;
         MP += (G % 4 == 2) ? 2 : 0;
@@ -317,6 +318,7 @@ void plan_batch(const scola_ctx *c, const std::vector<BoxGeom> &tiling_geo, int 
         const long long ng3 = (long long)g.ng * g.ng * g.ng;
         const long long np3 = (long long)(g.ng + 2 * G) * (g.ng + 2 * G) * (g.ng + 2 * G);
         add(bp.pch, bp.n_pch, b, n, kChunk);
+        add(bp.bch, bp.n_bch, b, block_count(g.nsc), 1);
         add(bp.tch, bp.n_tch, b, (long long)ntile * ntile * ntile, kChunk);
         add(bp.shch, bp.n_shch, b, np3 - ng3, kChunk);
         add(bp.mch, bp.n_mch, b, ng3, kChunk);
@@ -332,10 +334,11 @@ void plan_batch(const scola_ctx *c, const std::vector<BoxGeom> &tiling_geo, int 
         auto align64 = [](long long v) { return (v + 63) / 64 * 64; };
         P += n;
         M = align64(M + ng3);   // (the next box rounds up further)
-        MP = align64(MP + np3);
+        MP = (MP + np3 + 127) / 128 * 128;
         SH = align64(SH + np3 - ng3);
     }
     bp.pbeg.push_back((int)bp.n_pch);
+    bp.bbeg.push_back((int)bp.n_bch);
     bp.shbeg.push_back((int)bp.n_shch);
     bp.zbeg.push_back((int)bp.n_zit);
     bp.cbeg.push_back((int)bp.n_cit);
@@ -436,7 +439,7 @@ long long batch_bytes(const std::vector<BoxGeom> &geo, int G) {
         long long q = 64;
         while (q % g.ng) q += 64;
         bytes += 4 * 12 * n + 16 * n + 3 * 4 * 8 * nbe * nbe * nbe   // particles, sorted entries, keys
-                 + 2 * 4 * (ng3 + q) + 4 * (np3 + 66) + 4 * (np3 - ng3 + 64)   // meshes, shell
+                 + 2 * 4 * (ng3 + q) + 4 * (np3 + 130) + 4 * (np3 - ng3 + 64)   // meshes, shell
                  + 8 * (2 * n / kChunk + 2 * np3 / kChunk + ng3 / kChunk + 3 * g.ng * g.ng + 64);  // lists
     }
     return bytes;
@@ -458,6 +461,41 @@ scola_status bind_coefficients(scola_ctx *c, int first, int count) {
                        cudaMemcpyDeviceToDevice, c->stream));
     CK(cudaMemcpyAsync(c->coefL, c->all_coefL + 2 * (size_t)first, sizeof(float) * 2 * count,
                        cudaMemcpyDeviceToDevice, c->stream));
+    return SCOLA_OK;
+}
+
+// Textures of the bound boxes' padded potentials (FDA order 2) where every box allows one: padded
+// rows of a multiple of 4 cells (a plane is then a whole number of 32-byte texture pitches), and
+// planes of at most 2^16 cells (columns and their halves stay exact in the texture unit's
+// coordinates).  Otherwise, or where the driver refuses one, the interpolation uses plain loads.
+void drop_textures(scola_ctx *c) {
+    for (cudaTextureObject_t t : c->phi_tex_h) cudaDestroyTextureObject(t);
+    c->phi_tex_h.clear();
+    c->tex_ok = false;
+}
+
+scola_status bind_textures(scola_ctx *c) {
+    drop_textures(c);
+    if (c->prm.fda_order != 2) return SCOLA_OK;
+    cudaDeviceProp prop;
+    CK(cudaGetDeviceProperties(&prop, c->device));
+    for (const BoxDesc &B : c->boxes_h) {
+        const int S = B.Ng + 2 * B.gpad;
+        if (S % 4 != 0 || S * S > 65536 || S * S > prop.maxTexture2DLinear[0] ||
+            (size_t)S * S * sizeof(float) > (size_t)prop.maxTexture2DLinear[2] || prop.textureAlignment > 512)
+            return SCOLA_OK;
+    }
+    for (const BoxDesc &B : c->boxes_h) {
+        cudaTextureObject_t t = 0;
+        if (phi_texture(*c, B, &t) != cudaSuccess) {
+            cudaGetLastError();
+            drop_textures(c);
+            return SCOLA_OK;
+        }
+        c->phi_tex_h.push_back(t);
+    }
+    CS(put(c->phi_tex, c->phi_tex_h));
+    c->tex_ok = true;
     return SCOLA_OK;
 }
 
@@ -491,6 +529,7 @@ scola_status bind_batch(scola_ctx *c, int k, bool force = false) {
     }
     CS(put(c->boxes, bp.boxes));
     CS(put(c->pchunks, bp.pch));
+    CS(put(c->bchunks, bp.bch));
     CS(put(c->tchunks, bp.tch));
     CS(put(c->shchunks, bp.shch));
     CS(put(c->zitems, bp.zit));
@@ -506,6 +545,8 @@ scola_status bind_batch(scola_ctx *c, int k, bool force = false) {
     c->nboxes = count;
     c->boxes_h = bp.boxes;
     c->n_pchunks = (int)bp.n_pch;
+    c->n_bchunks = (int)bp.n_bch;
+    c->bbeg = bp.bbeg;
     c->n_tchunks = (int)bp.n_tch;
     c->n_shchunks = (int)bp.n_shch;
     c->n_zitems = (int)bp.n_zit;
@@ -547,6 +588,7 @@ scola_status bind_batch(scola_ctx *c, int k, bool force = false) {
     c->MP = bp.MP;
     c->SH = bp.SH;
     CS(bind_coefficients(c, first, count));
+    CS(bind_textures(c));
     c->bound_batch = k;
     return SCOLA_OK;
 }
@@ -868,7 +910,7 @@ scola_status build(scola_ctx *c, const std::vector<BoxGeom> &all_geo) {
 
     // every batch's layout (box descriptors kept; list lengths and arena sizes maxed)
     long long P = 0, M = 0, MP = 0, SH = 0, NK = 0, dep = 0;
-    long long L_pch = 0, L_tch = 0, L_shch = 0, L_zit = 0, L_cit = 0, L_mch = 0, L_ppch = 0, L_sbr = 0, L_tct = 0,
+    long long L_pch = 0, L_bch = 0, L_tch = 0, L_shch = 0, L_zit = 0, L_cit = 0, L_mch = 0, L_ppch = 0, L_sbr = 0, L_tct = 0,
               L_pl = 0, L_rx = 0, L_xp = 0;
     int max_count = 0;
     for (int k = 0; k < nbatch; ++k) {
@@ -883,6 +925,7 @@ scola_status build(scola_ctx *c, const std::vector<BoxGeom> &all_geo) {
         NK = std::max(NK, bp.NK);
         dep = std::max(dep, bp.dep_cells);
         L_pch = std::max(L_pch, bp.n_pch);
+        L_bch = std::max(L_bch, bp.n_bch);
         L_tch = std::max(L_tch, bp.n_tch);
         L_shch = std::max(L_shch, bp.n_shch);
         L_zit = std::max(L_zit, bp.n_zit);
@@ -905,6 +948,8 @@ scola_status build(scola_ctx *c, const std::vector<BoxGeom> &all_geo) {
     CS(upload(&c->all_boxes, c->all_boxes_h));
     CS(dev_alloc(&c->boxes, max_count));
     CS(dev_alloc(&c->pchunks, L_pch));
+    CS(dev_alloc(&c->bchunks, L_bch));
+    CS(dev_alloc(&c->phi_tex, max_count));
     CS(dev_alloc(&c->tchunks, L_tch));
     CS(dev_alloc(&c->shchunks, L_shch));
     CS(dev_alloc(&c->zitems, L_zit));
@@ -1115,13 +1160,13 @@ scola_status fill_light_cone_tables(scola_ctx *c) {
 // Restricts every work list to one box; restores on destruction.
 struct BoxView {
     scola_ctx *c;
-    Chunk *pch, *sh, *z, *cl, *mc, *sb;
-    int npch, nsh, nz, ncl, nmc, nsb;
+    Chunk *pch, *bch, *sh, *z, *cl, *mc, *sb;
+    int npch, nbch, nsh, nz, ncl, nmc, nsb;
     int view;
     BoxView(scola_ctx *cc, int b) : c(cc) {
         view = c->view_box;
         c->view_box = b;
-        pch = c->pchunks; sh = c->shchunks; z = c->zitems; cl = c->citems; mc = c->mchunks; sb = c->sbricks;
+        pch = c->pchunks; bch = c->bchunks; nbch = c->n_bchunks; sh = c->shchunks; z = c->zitems; cl = c->citems; mc = c->mchunks; sb = c->sbricks;
         npch = c->n_pchunks; nsh = c->n_shchunks; nz = c->n_zitems; ncl = c->n_citems;
         nmc = c->n_mchunks; nsb = c->n_sbricks;
         c->sbricks = sb + c->sbbeg[b];
@@ -1130,6 +1175,8 @@ struct BoxView {
         c->n_mchunks = c->mbeg[b + 1] - c->mbeg[b];
         c->pchunks = pch + c->pbeg[b];
         c->n_pchunks = c->pbeg[b + 1] - c->pbeg[b];
+        c->bchunks = bch + c->bbeg[b];
+        c->n_bchunks = c->bbeg[b + 1] - c->bbeg[b];
         c->shchunks = sh + c->shbeg[b];
         c->n_shchunks = c->shbeg[b + 1] - c->shbeg[b];
         c->zitems = z + c->zbeg[b];
@@ -1138,7 +1185,7 @@ struct BoxView {
         c->n_citems = c->cbeg[b + 1] - c->cbeg[b];
     }
     ~BoxView() {
-        c->pchunks = pch; c->shchunks = sh; c->zitems = z; c->citems = cl; c->mchunks = mc; c->sbricks = sb;
+        c->pchunks = pch; c->bchunks = bch; c->n_bchunks = nbch; c->shchunks = sh; c->zitems = z; c->citems = cl; c->mchunks = mc; c->sbricks = sb;
         c->n_pchunks = npch; c->n_shchunks = nsh; c->n_zitems = nz; c->n_citems = ncl;
         c->n_mchunks = nmc; c->n_sbricks = nsb;
         c->view_box = view;
@@ -1531,11 +1578,12 @@ void scola_destroy(scola_ctx *c) {
     if (c->stream) cudaStreamSynchronize(c->stream);
     else cudaDeviceSynchronize();
     if (c->evolve_exec) cudaGraphExecDestroy(c->evolve_exec);
+    drop_textures(c);
     if (c->have_plans) {
         cufftDestroy(c->plan_r2c);
         cufftDestroy(c->plan_c2r);
     }
-    void *ptrs[] = {c->boxes, c->all_boxes, c->all_coef, c->all_coefL, c->coef, c->coefL, c->tables, c->table_arena, c->pchunks, c->tchunks, c->shchunks,
+    void *ptrs[] = {c->boxes, c->all_boxes, c->all_coef, c->all_coefL, c->coef, c->coefL, c->tables, c->table_arena, c->pchunks, c->bchunks, c->phi_tex, c->tchunks, c->shchunks,
                     c->zitems, c->citems, c->mchunks, c->ppchunks, c->tc_tiles, c->tc_planes, c->rx_tiles, c->tri_boxes, c->xplanes, c->dev_err, c->ckpt, c->ckpt_phi, c->seg, c->fin,
                     c->adj, c->lamG, c->lam_phi_pad, c->adj_in, c->adj_out, c->lam_shell, c->lamPsi1,
                     c->lamPsi2, c->lam_phi1, c->lam_phi2, c->d2, c->lam_d2, c->part, c->dep_acc, c->kcount,

@@ -105,6 +105,43 @@ __device__ __forceinline__ void decode_local(int local, int n, int &i, int &j, i
     i = t / n;
 }
 
+// Blocks of 256 lattice sites for the kernels that gather from the mesh: 4 x (64 / z) x z sites
+// (x, y, z extents), z = 16 where that divides the box, else 8.  A block's stencils share more
+// cache lines than a run of 256 sites along z, and its state is still read in whole sectors.
+// Boxes that blocks would cover with more than an eighth of idle lanes (25 sites a side: 83 %)
+// keep the runs: block_z = 0.
+__host__ __device__ inline int block_tiles(int Nsc, int bz) {
+    const int by = 64 / bz;
+    return ((Nsc + 3) / 4) * ((Nsc + by - 1) / by) * ((Nsc + bz - 1) / bz);
+}
+__host__ __device__ inline int block_z(int Nsc) {
+    const int bz = Nsc % 16 == 0 ? 16 : 8;
+    return 8LL * 256 * block_tiles(Nsc, bz) <= 9LL * Nsc * Nsc * Nsc ? bz : 0;
+}
+__host__ __device__ inline int block_count(int Nsc) {
+    const int bz = block_z(Nsc);
+    return bz ? block_tiles(Nsc, bz) : (Nsc * Nsc * Nsc + 255) / 256;
+}
+// Site t (0 .. 255) of block q of a box; false beyond the lattice.
+__device__ __forceinline__ bool block_site(int q, int t, int Nsc, int &i, int &j, int &k) {
+    const int bz = block_z(Nsc);
+    if (bz == 0) {
+        const int local = q * 256 + t;
+        k = local % Nsc;
+        const int r = local / Nsc;
+        j = r % Nsc;
+        i = r / Nsc;
+        return i < Nsc;
+    }
+    const int by = 64 / bz;
+    const int nz = (Nsc + bz - 1) / bz, ny = (Nsc + by - 1) / by;
+    const int r = q / nz;
+    k = (q - r * nz) * bz + (t & (bz - 1));
+    j = (r % ny) * by + ((t & 63) / bz);
+    i = (r / ny) * 4 + (t >> 6);
+    return i < Nsc && j < Nsc && k < Nsc;
+}
+
 // Per-tile final scale factors: box b's FP32 coefficients at force evaluation k (see Ctx::coef),
 // or null when the launch uses uniform scalars.
 __device__ __forceinline__ const float *box_coef(const float *coef, int box, int k, int nk) {

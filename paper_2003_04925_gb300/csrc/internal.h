@@ -141,6 +141,15 @@ struct Ctx {
     DstTable *tables = nullptr;
     float *table_arena = nullptr;
     Chunk *pchunks = nullptr;  int n_pchunks = 0;     // box particles
+    // box particles in blocks of 4 x (64 / z) x z lattice sites, z = 16 or 8 (block_z): the
+    // interpolation kernels
+    Chunk *bchunks = nullptr;  int n_bchunks = 0;
+    std::vector<int> bbeg;
+    // FDA order 2, every padded row a multiple of 4 cells: a 2D texture of each box's padded
+    // potential (rows: x planes, columns: (y, z)), for the interpolation's 2 x 2 gathers
+    std::vector<cudaTextureObject_t> phi_tex_h;       // the bound batch's
+    cudaTextureObject_t *phi_tex = nullptr;
+    bool tex_ok = false;
     Chunk *tchunks = nullptr;  int n_tchunks = 0;     // tile particles (scatter)
     Chunk *shchunks = nullptr; int n_shchunks = 0;    // shell cells
     Chunk *zitems = nullptr;   int n_zitems = 0;      // z-pencil tiles
@@ -303,6 +312,7 @@ cudaError_t launch_poisson_buffers(Ctx &c, const float *in, float *w1, float *w2
 cudaError_t launch_poisson(Ctx &c);
 cudaError_t launch_poisson_pass(Ctx &c, int pass);
 // F = D1 x gradient of the stored potential Phi / D1
+cudaError_t phi_texture(Ctx &c, const BoxDesc &B, cudaTextureObject_t *out);
 cudaError_t launch_interp(Ctx &c, const float *s, long long stride, float *F, float D1);
 cudaError_t launch_scaled_copy(Ctx &c, const float *in, float *out, long long n, float a);
 // count_keys: also count the sorted deposit's keys of the drifted particles (into cleared

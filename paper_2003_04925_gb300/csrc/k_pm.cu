@@ -203,9 +203,18 @@ k_dst(const BoxDesc *__restrict__ boxes, const DstTable *__restrict__ tables,
 // CIC corners, CIC-interpolated.  The mesh coordinate is clamped to [-N_ghost,
 // Ng + N_ghost - 1] and the lower corner capped at Ng + N_ghost - 2 (the gradient exists on
 // the grid padded by N_ghost, Sec. 3.4.2).
-template <int ORDER>
+//
+// The 32 gathers of order 2 are bound by the L1's wavefronts (78 % of their peak rate at 64 boxes
+// of 96^3 cells, DRAM 21 %): neighbouring particles drift to other rows and lines.  Where the box
+// has a texture of its padded potential (kTex), 24 of the 32 values come as six 2 x 2 gathers in
+// the (x, z) plane through the texture pipe, which runs beside the load pipe; the eight outer z
+// values stay plain loads (texture gathers alone saturate at 16 cycles a warp instruction).  Force
+// interpolation alone (k_interp), plain / with textures, each in blocks of sites: 64 boxes of 96^3
+// cells at 2:1 247 / 180 us, 64 of 72-96 at 1:1 844 / 603 us, 16 of 192^3 573 / 376 us.
+template <int ORDER, bool kTex>
 __device__ __forceinline__ void interpolate_force(const BoxDesc &B, const float *__restrict__ phi,
-                                                  const int b[3], const float s[3], float F[3]) {
+                                                  cudaTextureObject_t tex, const int b[3], const float s[3],
+                                                  float F[3]) {
     const int Ng = B.Ng, G = B.gpad, ng = Fda<ORDER>::ng;
     int i0[3];
     float w[3][2];
@@ -224,23 +233,51 @@ __device__ __forceinline__ void interpolate_force(const BoxDesc &B, const float 
     const float *P = phi + B.pp_off + ((long long)(i0[0] + G) * S1 + (i0[1] + G)) * S1 + (i0[2] + G);
     if (ORDER == 2) {
         float core[2][2][2], xm[2][2], xp[2][2], ym[2][2], yp[2][2], zm[2][2], zp[2][2];
-#pragma unroll
-        for (int a = 0; a < 2; ++a)
-#pragma unroll
-            for (int bb = 0; bb < 2; ++bb)
-#pragma unroll
-                for (int c = 0; c < 2; ++c) core[a][bb][c] = __ldg(P + a * S2 + bb * S1 + c);
-#pragma unroll
-        for (int p = 0; p < 2; ++p)
+        // the texture's rows are one plane of S^2 cells long and start 2 cells before the plane
+        // (phi_texture): the last two cells of a plane, reached from the uppermost (y, z) corner
+        // alone, lie beyond its width
+        if (kTex && !(i0[1] == Ng - 1 && i0[2] == Ng - 1)) {
+            const float col = (float)((i0[1] + G) * (int)S1 + (i0[2] + G) + 3), row = (float)(i0[0] + G + 1);
+            // texels (x, x + 1) x (z, z + 1) at row `dx` and z-row `dy` from the lower corner, in the
+            // order (x + 1, z), (x + 1, z + 1), (x, z + 1), (x, z)
+            auto quad = [&](int dx, int dy) {
+                return tex2Dgather<float4>(tex, col + (float)(dy * (int)S1), row + (float)dx, 0);
+            };
 #pragma unroll
             for (int q = 0; q < 2; ++q) {
-                xm[p][q] = __ldg(P - S2 + p * S1 + q);
-                xp[p][q] = __ldg(P + 2 * S2 + p * S1 + q);
-                ym[p][q] = __ldg(P + p * S2 - S1 + q);
-                yp[p][q] = __ldg(P + p * S2 + 2 * S1 + q);
-                zm[p][q] = __ldg(P + p * S2 + q * S1 - 1);
-                zp[p][q] = __ldg(P + p * S2 + q * S1 + 2);
+                const float4 lo = quad(-1, q), hi = quad(1, q);
+                xm[q][0] = lo.w, xm[q][1] = lo.z, core[0][q][0] = lo.x, core[0][q][1] = lo.y;
+                core[1][q][0] = hi.w, core[1][q][1] = hi.z, xp[q][0] = hi.x, xp[q][1] = hi.y;
             }
+            const float4 below = quad(0, -1), above = quad(0, 2);
+            ym[0][0] = below.w, ym[0][1] = below.z, ym[1][0] = below.x, ym[1][1] = below.y;
+            yp[0][0] = above.w, yp[0][1] = above.z, yp[1][0] = above.x, yp[1][1] = above.y;
+#pragma unroll
+            for (int p = 0; p < 2; ++p)
+#pragma unroll
+                for (int q = 0; q < 2; ++q) {
+                    zm[p][q] = __ldg(P + p * S2 + q * S1 - 1);
+                    zp[p][q] = __ldg(P + p * S2 + q * S1 + 2);
+                }
+        } else {
+#pragma unroll
+            for (int a = 0; a < 2; ++a)
+#pragma unroll
+                for (int bb = 0; bb < 2; ++bb)
+#pragma unroll
+                    for (int c = 0; c < 2; ++c) core[a][bb][c] = __ldg(P + a * S2 + bb * S1 + c);
+#pragma unroll
+            for (int p = 0; p < 2; ++p)
+#pragma unroll
+                for (int q = 0; q < 2; ++q) {
+                    xm[p][q] = __ldg(P - S2 + p * S1 + q);
+                    xp[p][q] = __ldg(P + 2 * S2 + p * S1 + q);
+                    ym[p][q] = __ldg(P + p * S2 - S1 + q);
+                    yp[p][q] = __ldg(P + p * S2 + 2 * S1 + q);
+                    zm[p][q] = __ldg(P + p * S2 + q * S1 - 1);
+                    zp[p][q] = __ldg(P + p * S2 + q * S1 + 2);
+                }
+        }
         float fx = 0.0f, fy = 0.0f, fz = 0.0f;
 #pragma unroll
         for (int p = 0; p < 2; ++p)
@@ -286,27 +323,27 @@ __device__ __forceinline__ void interpolate_force(const BoxDesc &B, const float 
     for (int a = 0; a < 3; ++a) F[a] = acc[a] * B.inv_dg;
 }
 
-template <int ORDER>
+template <int ORDER, bool kTex>
 __global__ void __launch_bounds__(kChunk)
-k_interp(const BoxDesc *__restrict__ boxes, const Chunk *__restrict__ chunks,
-         const float *__restrict__ s, long long stride, const float *__restrict__ phi, float D1,
-         float *__restrict__ F) {
-    const Chunk ch = chunks[blockIdx.x];
+k_interp(const BoxDesc *__restrict__ boxes, const Chunk *__restrict__ blocks,
+         const float *__restrict__ s, long long stride, const float *__restrict__ phi,
+         const cudaTextureObject_t *__restrict__ tex, float D1, float *__restrict__ F) {
+    const Chunk ch = blocks[blockIdx.x];
     const BoxDesc &B = boxes[ch.box];
-    const int Nsc = B.Nsc;
-    const int local = ch.start + threadIdx.x;
-    if (local >= Nsc * Nsc * Nsc) return;
-    const long long gi = B.p_off + local;
     int b[3];
-    decode_local(local, Nsc, b[0], b[1], b[2]);
+    if (!block_site(ch.start, threadIdx.x, B.Nsc, b[0], b[1], b[2])) return;
+    const long long gi = B.p_off + (b[0] * B.Nsc + b[1]) * B.Nsc + b[2];
     float sv[3] = {s[gi], s[stride + gi], s[2 * stride + gi]};
     float f[3];
-    interpolate_force<ORDER>(B, phi, b, sv, f);
+    interpolate_force<ORDER, kTex>(B, phi, kTex ? tex[ch.box] : 0, b, sv, f);
     F[gi] = D1 * f[0];
     F[stride + gi] = D1 * f[1];
     F[2 * stride + gi] = D1 * f[2];
 }
 
+// (In runs of 256 sites along z and with plain gathers: its 72 bytes of state a particle set the
+// pace until the late steps of dense boxes, and over a run's evaluations on 64 boxes of 96^3 cells
+// it takes 202 us a launch against 243-247 us with texture gathers, 215 us in blocks of sites.)
 template <int ORDER>
 __global__ void __launch_bounds__(kChunk, 5)
 k_kick_drift(const BoxDesc *__restrict__ boxes, const Chunk *__restrict__ chunks,
@@ -338,7 +375,7 @@ k_kick_drift(const BoxDesc *__restrict__ boxes, const Chunk *__restrict__ chunks
             p2[a] = __ldg(part + (9 + a) * P + gi);
         }
         float F[3];
-        interpolate_force<ORDER>(B, phi, b, s, F);
+        interpolate_force<ORDER, false>(B, phi, 0, b, s, F);
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
             p[a] = fmaf(kd.kF, F[a], fmaf(kd.k1, p1[a], fmaf(kd.k2, p2[a], p[a])));
@@ -481,14 +518,35 @@ cudaError_t launch_poisson_pass(Ctx &c, int pass) {
     }
 }
 
+// (with texture gathers at order 2 where the boxes have them)
 cudaError_t launch_interp(Ctx &c, const float *s, long long stride, float *F, float D1) {
-    switch (c.prm.fda_order) {
-        case 4: k_interp<4><<<c.n_pchunks, kChunk, 0, c.stream>>>(c.boxes, c.pchunks, s, stride, c.phi, D1, F); break;
-        case 6: k_interp<6><<<c.n_pchunks, kChunk, 0, c.stream>>>(c.boxes, c.pchunks, s, stride, c.phi, D1, F); break;
-        default: k_interp<2><<<c.n_pchunks, kChunk, 0, c.stream>>>(c.boxes, c.pchunks, s, stride, c.phi, D1, F);
-    }
+#define SCOLA_INTERP(ORDER, TEX)                                                                          \
+    k_interp<ORDER, TEX><<<c.n_bchunks, kChunk, 0, c.stream>>>(c.boxes, c.bchunks, s, stride, c.phi, c.phi_tex, D1, F)
+    if (c.prm.fda_order == 4) SCOLA_INTERP(4, false);
+    else if (c.prm.fda_order == 6) SCOLA_INTERP(6, false);
+    else if (c.tex_ok) SCOLA_INTERP(2, true);
+    else SCOLA_INTERP(2, false);
+#undef SCOLA_INTERP
     ++c.launches;
     return cudaGetLastError();
+}
+
+// A 2D texture of a box's padded potential: row x, column 2 + y S + z, the rows S^2 cells apart.
+// The box starts 2 cells past a multiple of 128 cells (plan_batch), where the texture begins.
+cudaError_t phi_texture(Ctx &c, const BoxDesc &B, cudaTextureObject_t *out) {
+    const long long S = B.Ng + 2 * B.gpad;
+    cudaResourceDesc r = {};
+    r.resType = cudaResourceTypePitch2D;
+    r.res.pitch2D.devPtr = c.phi + (B.pp_off - 2);
+    r.res.pitch2D.desc = cudaCreateChannelDesc<float>();
+    r.res.pitch2D.width = (size_t)(S * S);
+    r.res.pitch2D.height = (size_t)S;
+    r.res.pitch2D.pitchInBytes = (size_t)(S * S) * sizeof(float);
+    cudaTextureDesc t = {};
+    t.addressMode[0] = t.addressMode[1] = cudaAddressModeClamp;
+    t.filterMode = cudaFilterModePoint;
+    t.readMode = cudaReadModeElementType;
+    return cudaCreateTextureObject(out, &r, &t, nullptr);
 }
 
 namespace {
