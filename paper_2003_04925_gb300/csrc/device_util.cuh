@@ -275,4 +275,49 @@ __device__ __forceinline__ int wrap(int v, int n) {
     return v < 0 ? v + n : v;
 }
 
+// The same for v within one period of [0, n) (indices next to a position in the box): a compare
+// and an add; anything further out takes the remainder.
+__device__ __forceinline__ int wrap_near(int v, int n) {
+    if (v < 0) v += n;
+    if (v >= n) v -= n;
+    return (unsigned)v < (unsigned)n ? v : wrap(v, n);
+}
+
+// Periodic CIC deposit of one particle per lane on an N^3 grid of 2^-32 fixed-point counts: lower
+// corner i0 (not wrapped), fractions f; every lane of the warp calls it (valid or not).
+// kMerge, for grids of one cell per particle spacing: consecutive lanes hold Lagrangian
+// z-neighbours, and where a lane's lower corner is its left neighbour's moved one cell up in z the
+// neighbour's four upper-z weights join its own lower-z ones and the neighbour skips those atomics
+// (integer sums: the same totals).
+template <bool kMerge>
+__device__ __forceinline__ void periodic_deposit(unsigned long long *acc, int N, const int (&i0)[3], const float (&f)[3],
+                                                 bool valid) {
+    bool take = false, give = false;
+    if (kMerge) {
+        const int lane = threadIdx.x & 31, key = valid ? i0[2] : 0x40000000;
+        const int px = __shfl_up_sync(0xffffffffu, i0[0], 1), py = __shfl_up_sync(0xffffffffu, i0[1], 1),
+                  pz = __shfl_up_sync(0xffffffffu, key, 1);
+        take = valid && lane > 0 && px == i0[0] && py == i0[1] && pz + 1 == i0[2];
+        give = __shfl_down_sync(0xffffffffu, take ? 1 : 0, 1) && lane < 31;
+    }
+    const int z0 = wrap_near(i0[2], N), z1 = z0 + 1 == N ? 0 : z0 + 1;
+#pragma unroll
+    for (int dx = 0; dx < 2; ++dx) {
+        const float wx = dx ? f[0] : 1.0f - f[0];
+#pragma unroll
+        for (int dy = 0; dy < 2; ++dy) {
+            const float wxy = wx * (dy ? f[1] : 1.0f - f[1]);
+            unsigned long long lo = weight_to_fixed(wxy * (1.0f - f[2])), up = weight_to_fixed(wxy * f[2]);
+            if (kMerge) {
+                const unsigned long long left = __shfl_up_sync(0xffffffffu, up, 1);
+                if (take) lo += left;
+            }
+            if (!valid) continue;
+            unsigned long long *row = acc + ((long long)wrap_near(i0[0] + dx, N) * N + wrap_near(i0[1] + dy, N)) * N;
+            atomicAdd(row + z0, lo);
+            if (!give) atomicAdd(row + z1, up);
+        }
+    }
+}
+
 }  // namespace scola

@@ -140,7 +140,13 @@ __global__ void k_density_vjp(const float *__restrict__ x, long long n, int Np, 
             i0[a] = (int)fl;
             f[a] = u - fl;
         }
-        const long long NN = (long long)Np * Np;
+        long long row[2][2];                       // the four (x, y) corner rows
+        const int z[2] = {wrap_near(i0[2], Np), wrap_near(i0[2] + 1, Np)};
+#pragma unroll
+        for (int dx = 0; dx < 2; ++dx)
+#pragma unroll
+            for (int dy = 0; dy < 2; ++dy)
+                row[dx][dy] = ((long long)wrap_near(i0[0] + dx, Np) * Np + wrap_near(i0[1] + dy, Np)) * Np;
         float lam[3] = {0.f, 0.f, 0.f};
 #pragma unroll
         for (int dx = 0; dx < 2; ++dx)
@@ -150,8 +156,7 @@ __global__ void k_density_vjp(const float *__restrict__ x, long long n, int Np, 
                 for (int dz = 0; dz < 2; ++dz) {
                     const float wx = dx ? f[0] : 1.f - f[0], wy = dy ? f[1] : 1.f - f[1],
                                 wz = dz ? f[2] : 1.f - f[2];
-                    const float v = lam_delta[wrap(i0[0] + dx, Np) * NN + (long long)wrap(i0[1] + dy, Np) * Np +
-                                              wrap(i0[2] + dz, Np)];
+                    const float v = __ldg(lam_delta + row[dx][dy] + z[dz]);
                     lam[0] += (dx ? 1.f : -1.f) * wy * wz * v;
                     lam[1] += wx * (dy ? 1.f : -1.f) * wz * v;
                     lam[2] += wx * wy * (dz ? 1.f : -1.f) * v;

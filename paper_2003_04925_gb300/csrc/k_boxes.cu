@@ -138,36 +138,24 @@ k_box_ids(const BoxDesc *__restrict__ boxes, const Chunk *__restrict__ chunks, i
     out[B.p_off + local] = box_particle_gid(B, Np, Ntile, bi, bj, bk);
 }
 
+// (256^3 particles at a = 1: 472 us, 486 us with a remainder per corner index and eight atomics a
+// particle: the L2 rate of the 64-bit atomics, 2.8e11 a second, sets the pace.)
 __global__ void k_density_deposit(const float *__restrict__ x, long long n, int N, float inv_d,
                                   unsigned long long *__restrict__ acc) {
-    for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < n;
-         idx += (long long)gridDim.x * blockDim.x) {
-        int i0[3];
-        float f[3];
+    // (whole warps: the deposit shares weights between lanes)
+    for (long long base = blockIdx.x * (long long)blockDim.x; base < n; base += (long long)gridDim.x * blockDim.x) {
+        const long long idx = base + threadIdx.x;
+        const bool valid = idx < n;
+        int i0[3] = {0, 0, 0};
+        float f[3] = {0.0f, 0.0f, 0.0f};
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-            const float u = x[idx * 3 + a] * inv_d - 0.5f;
+            const float u = valid ? x[idx * 3 + a] * inv_d - 0.5f : 0.0f;
             const float fl = floorf(u);
             i0[a] = (int)fl;
             f[a] = u - fl;
         }
-        const long long NN = (long long)N * N;
-#pragma unroll
-        for (int dx = 0; dx < 2; ++dx) {
-            const long long ix = wrap(i0[0] + dx, N);
-            const float wx = dx ? f[0] : 1.0f - f[0];
-#pragma unroll
-            for (int dy = 0; dy < 2; ++dy) {
-                const long long iy = wrap(i0[1] + dy, N);
-                const float wxy = wx * (dy ? f[1] : 1.0f - f[1]);
-#pragma unroll
-                for (int dz = 0; dz < 2; ++dz) {
-                    const long long iz = wrap(i0[2] + dz, N);
-                    const float w = wxy * (dz ? f[2] : 1.0f - f[2]);
-                    atomicAdd(acc + ix * NN + iy * N + iz, weight_to_fixed(w));
-                }
-            }
-        }
+        periodic_deposit<true>(acc, N, i0, f, valid);
     }
 }
 

@@ -30,11 +30,12 @@ namespace scola {
 
 namespace {
 
+// (Np <= 1024: 32-bit indices)
 __device__ __forceinline__ void gid_coords(long long gid, int Np, int g[3]) {
-    g[2] = (int)(gid % Np);
-    const long long t = gid / Np;
-    g[1] = (int)(t % Np);
-    g[0] = (int)(t / Np);
+    const unsigned i = (unsigned)gid, t = i / (unsigned)Np, x = t / (unsigned)Np;
+    g[2] = (int)(i - t * (unsigned)Np);
+    g[1] = (int)(t - x * (unsigned)Np);
+    g[0] = (int)x;
 }
 
 // Mesh coordinate of a particle: u = x / dg - 1/2 with x = (g + 1/2) dq + s.
@@ -55,38 +56,25 @@ __global__ void k_tc_init(float *__restrict__ part, const float *__restrict__ ps
     }
 }
 
+template <bool kMerge>
 __global__ void k_tc_deposit(const float *__restrict__ part, long long N3, int Np, int Ngf, float q2u,
                              float inv_dg, unsigned long long *__restrict__ acc) {
-    const long long NN = (long long)Ngf * Ngf;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N3;
-         i += (long long)gridDim.x * blockDim.x) {
+    // (whole warps: the deposit may share weights between lanes)
+    for (long long base = blockIdx.x * (long long)blockDim.x; base < N3; base += (long long)gridDim.x * blockDim.x) {
+        const long long i = base + threadIdx.x;
+        const bool valid = i < N3;
         int g[3];
-        gid_coords(i, Np, g);
+        gid_coords(valid ? i : 0, Np, g);
         int i0[3];
         float f[3];
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-            const float u = mesh_u(g[a], part[a * N3 + i], q2u, inv_dg);
+            const float u = mesh_u(g[a], valid ? part[a * N3 + i] : 0.0f, q2u, inv_dg);
             const float fl = floorf(u);
             i0[a] = (int)fl;
             f[a] = u - fl;
         }
-#pragma unroll
-        for (int dx = 0; dx < 2; ++dx) {
-            const long long cx = wrap(i0[0] + dx, Ngf);
-            const float wx = dx ? f[0] : 1.0f - f[0];
-#pragma unroll
-            for (int dy = 0; dy < 2; ++dy) {
-                const long long cy = wrap(i0[1] + dy, Ngf);
-                const float wxy = wx * (dy ? f[1] : 1.0f - f[1]);
-#pragma unroll
-                for (int dz = 0; dz < 2; ++dz) {
-                    const long long cz = wrap(i0[2] + dz, Ngf);
-                    const float w = wxy * (dz ? f[2] : 1.0f - f[2]);
-                    atomicAdd(acc + cx * NN + cy * Ngf + cz, weight_to_fixed(w));
-                }
-            }
-        }
+        periodic_deposit<kMerge>(acc, Ngf, i0, f, valid);
     }
 }
 
@@ -114,7 +102,7 @@ k_tc_kick_drift(float *__restrict__ part, const float *__restrict__ psi1, const 
         p2[a] = __ldg(psi2 + a * N3 + i);
     }
     // wrapped indices i0 - 1 .. i0 + 2 per axis and the CIC weights
-    long long ix[4], iy[4], iz[4];
+    int ix[4], iy[4], iz[4];                       // (at most 2^30 cells)
     float w[3][2];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
@@ -126,7 +114,7 @@ k_tc_kick_drift(float *__restrict__ part, const float *__restrict__ psi1, const 
         w[a][1] = f;
 #pragma unroll
         for (int o = 0; o < 4; ++o) {
-            const long long v = wrap(i0 - 1 + o, Ngf);
+            const int v = wrap_near(i0 - 1 + o, Ngf);
             if (a == 0) ix[o] = v * Ngf * Ngf;
             if (a == 1) iy[o] = v * Ngf;
             if (a == 2) iz[o] = v;
@@ -237,8 +225,13 @@ cudaError_t launch_tc_init(Ctx &c) {
 
 cudaError_t launch_tc_deposit(Ctx &c) {
     const int ratio = c.tc_ng / c.Np;
-    k_tc_deposit<<<grid_of(c.N3, 256), 256, 0, c.stream>>>(c.tc_part, c.N3, c.Np, c.tc_ng, (float)ratio,
-                                                           (float)(c.tc_ng / c.L), c.tc_acc);
+    // lanes share weights on grids of one cell per particle (finer ones leave neighbours apart)
+    if (ratio == 1)
+        k_tc_deposit<true><<<grid_of(c.N3, 256), 256, 0, c.stream>>>(c.tc_part, c.N3, c.Np, c.tc_ng, (float)ratio,
+                                                                     (float)(c.tc_ng / c.L), c.tc_acc);
+    else
+        k_tc_deposit<false><<<grid_of(c.N3, 256), 256, 0, c.stream>>>(c.tc_part, c.N3, c.Np, c.tc_ng, (float)ratio,
+                                                                      (float)(c.tc_ng / c.L), c.tc_acc);
     ++c.launches;
     return cudaGetLastError();
 }
