@@ -39,7 +39,15 @@ struct BoxGeom {                         // one box of the tiling: Np,sCOLA, Ng,
     int nsc, ng, nbuf;
 };
 
+struct StageGraph {                      // a full-box stage's launches as a graph (run_graphed)
+    cudaGraphExec_t exec = nullptr;
+    long long kernels = 0;
+    int runs = 0;
+    bool refused = false;
+};
+
 struct scola_ctx : public Ctx {
+    StageGraph lpt_graph, tcola_graph;
     std::vector<double> a_final;         // per-tile final scale factors (empty: a_f for all)
     float *all_coef = nullptr, *all_coefL = nullptr;   // every context box's coefficients
     std::vector<BoxGeom> tiling_geo;     // every box of the tiling
@@ -1004,16 +1012,53 @@ scola_status build(scola_ctx *c, const std::vector<BoxGeom> &all_geo) {
     return SCOLA_OK;
 }
 
+// Runs a fixed sequence of launches on the context stream: the first time as it is, afterwards as
+// a CUDA graph captured on the second call (a context used once pays nothing for it), unless the
+// caller's stream is itself being captured.  The full-box stages are ~50 launches of a few
+// microseconds each: 128^3 initial conditions take 332 us as a graph, 431 us launch by launch.
+template <typename Body>
+scola_status run_graphed(scola_ctx *c, StageGraph &G, Body body) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(c->stream, &cap) != cudaSuccess) {
+        cudaGetLastError();
+        cap = cudaStreamCaptureStatusActive;
+    }
+    if (G.runs++ == 0 || G.refused || cap != cudaStreamCaptureStatusNone) return body();
+    if (!G.exec) {
+        const cudaStream_t user = c->stream;
+        const long long before = c->launches;
+        cudaGraph_t graph = nullptr;
+        CK(cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal));
+        c->stream = c->cap_stream;
+        const bool fft = cufftSetStream(c->plan_r2c, c->stream) == CUFFT_SUCCESS &&
+                         cufftSetStream(c->plan_c2r, c->stream) == CUFFT_SUCCESS;
+        const scola_status st = fft ? body() : SCOLA_ERR_CUDA;
+        cudaError_t e = cudaStreamEndCapture(c->cap_stream, &graph);
+        c->stream = user;
+        CF(cufftSetStream(c->plan_r2c, user));
+        CF(cufftSetStream(c->plan_c2r, user));
+        if (st == SCOLA_OK && e == cudaSuccess) e = cudaGraphInstantiate(&G.exec, graph, 0);
+        if (graph) cudaGraphDestroy(graph);
+        G.kernels = c->launches - before;
+        c->launches = before;
+        if (st != SCOLA_OK || e != cudaSuccess) {              // keep launching one by one
+            cudaGetLastError();
+            G.exec = nullptr;
+            G.refused = true;
+            return body();
+        }
+    }
+    CK(cudaGraphLaunch(G.exec, c->stream));
+    c->launches += G.kernels;
+    return SCOLA_OK;
+}
+
 // A.1-A.2 on the full box into the context's grids.
-scola_status run_lpt(scola_ctx *c, const float *w, float *delta_out) {
+scola_status lpt_stage(scola_ctx *c, const float *w) {
     const float invN3 = (float)(1.0 / (double)c->N3);
     CT(cufftExecR2C(c->plan_r2c, const_cast<cufftReal *>(reinterpret_cast<const cufftReal *>(w)), c->ck));
     CK(launch_colour(*c, c->ck));
     const size_t cbytes = sizeof(cufftComplex) * (size_t)c->Np * c->Np * (c->Np / 2 + 1);
-    if (delta_out) {
-        CK(cudaMemcpyAsync(c->ct, c->ck, cbytes, cudaMemcpyDeviceToDevice, c->stream));
-        CT(cufftExecC2R(c->plan_c2r, c->ct, delta_out));
-    }
     CK(launch_inv_laplacian(*c, c->ck, c->cp, 1.0f));
     CK(cudaMemcpyAsync(c->ct, c->cp, cbytes, cudaMemcpyDeviceToDevice, c->stream));
     CT(cufftExecC2R(c->plan_c2r, c->ct, c->phi1));
@@ -1022,7 +1067,6 @@ scola_status run_lpt(scola_ctx *c, const float *w, float *delta_out) {
         // Zel'dovich frame: no second-order potential or displacements
         CK(cudaMemsetAsync(c->phi2, 0, sizeof(float) * (size_t)c->N3, c->stream));
         CK(cudaMemsetAsync(c->psi2, 0, sizeof(float) * 3 * (size_t)c->N3, c->stream));
-            c->lpt_done = true;
         return SCOLA_OK;
     }
     for (int a = 0; a < 3; ++a) {
@@ -1040,9 +1084,29 @@ scola_status run_lpt(scola_ctx *c, const float *w, float *delta_out) {
     CK(launch_inv_laplacian(*c, c->ct, c->ct, invN3));
     CT(cufftExecC2R(c->plan_c2r, c->ct, c->phi2));
     CK(launch_gradient(*c, c->phi2, c->psi2));
-    c->lpt_done = true;
     return SCOLA_OK;
 }
+
+// The stage for white noise w, and the initial density if asked for (from the coloured spectrum,
+// which the stage leaves in ck).  As a graph the stage reads its noise from g[0], so w is copied
+// there first: up to 256^3 that costs less than the launches it saves.
+scola_status run_lpt(scola_ctx *c, const float *w, float *delta_out) {
+    if (c->Np <= 256 && c->lpt_graph.runs > 0) {
+        CK(cudaMemcpyAsync(c->g[0], w, sizeof(float) * (size_t)c->N3, cudaMemcpyDeviceToDevice, c->stream));
+        CS(run_graphed(c, c->lpt_graph, [&]() { return lpt_stage(c, c->g[0]); }));
+    } else {
+        ++c->lpt_graph.runs;
+        CS(lpt_stage(c, w));
+    }
+    c->lpt_done = true;
+    if (delta_out) {
+        const size_t cbytes = sizeof(cufftComplex) * (size_t)c->Np * c->Np * (c->Np / 2 + 1);
+        CK(cudaMemcpyAsync(c->ct, c->ck, cbytes, cudaMemcpyDeviceToDevice, c->stream));
+        CT(cufftExecC2R(c->plan_c2r, c->ct, delta_out));
+    }
+    return SCOLA_OK;
+}
+
 
 KickDrift kick_drift_coefficients(const TimeTable &t, int k) {
     const int n = (int)t.alpha.size();
@@ -1072,7 +1136,6 @@ KickDrift forward_kick(const TimeTable &t, int k) {
 scola_status run_tcola(scola_ctx *c, bool record) {
     CS(tcola_alloc(c));
     CK(cudaEventRecord(c->tc_ev[0], c->stream));
-    CK(launch_tc_init(*c));
     const int n = (int)c->tt.alpha.size();
     // profiling mode: events between the stages of every force evaluation
     const bool prof = c->profiling;
@@ -1083,19 +1146,26 @@ scola_status run_tcola(scola_ctx *c, bool record) {
     auto mark = [&](int k, int q) -> cudaError_t {
         return prof ? cudaEventRecord(c->tc_prof_ev[5 * k + q], c->stream) : cudaSuccess;
     };
-    for (int k = 0; k <= n; ++k) {
-        float *delta = record && c->rec_delta ? c->rec_delta + (size_t)k * c->tc_n3 : c->tc_delta;
-        float *phi = record && c->rec_phi ? c->rec_phi + (size_t)k * c->tc_n3 : c->tc_phi;
-        CK(mark(k, 0));
-        CK(launch_tc_deposit(*c));
-        CK(mark(k, 1));
-        CK(launch_tc_density(*c, delta));
-        CK(mark(k, 2));
-        CK(launch_tc_poisson(*c, delta, phi));
-        CK(mark(k, 3));
-        CK(launch_tc_kick_drift(*c, phi, kick_drift_coefficients(c->tt, k)));
-        CK(mark(k, 4));
-    }
+    auto evolve = [&]() -> scola_status {
+        CK(launch_tc_init(*c));
+        for (int k = 0; k <= n; ++k) {
+            float *delta = record && c->rec_delta ? c->rec_delta + (size_t)k * c->tc_n3 : c->tc_delta;
+            float *phi = record && c->rec_phi ? c->rec_phi + (size_t)k * c->tc_n3 : c->tc_phi;
+            CK(mark(k, 0));
+            CK(launch_tc_deposit(*c));
+            CK(mark(k, 1));
+            CK(launch_tc_density(*c, delta));
+            CK(mark(k, 2));
+            CK(launch_tc_poisson(*c, delta, phi));
+            CK(mark(k, 3));
+            CK(launch_tc_kick_drift(*c, phi, kick_drift_coefficients(c->tt, k)));
+            CK(mark(k, 4));
+        }
+        return SCOLA_OK;
+    };
+    // (the same launches on the same arrays every run: a graph, but for the records and events)
+    if (record || prof) CS(evolve());
+    else CS(run_graphed(c, c->tcola_graph, evolve));
     c->tc_profiled = prof;
     CK(cudaEventRecord(c->tc_ev[1], c->stream));
     c->tc_timed = true;
@@ -1578,6 +1648,8 @@ void scola_destroy(scola_ctx *c) {
     if (c->stream) cudaStreamSynchronize(c->stream);
     else cudaDeviceSynchronize();
     if (c->evolve_exec) cudaGraphExecDestroy(c->evolve_exec);
+    if (c->lpt_graph.exec) cudaGraphExecDestroy(c->lpt_graph.exec);
+    if (c->tcola_graph.exec) cudaGraphExecDestroy(c->tcola_graph.exec);
     drop_textures(c);
     if (c->have_plans) {
         cufftDestroy(c->plan_r2c);
