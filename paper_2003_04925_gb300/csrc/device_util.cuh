@@ -98,11 +98,28 @@ __device__ __forceinline__ float boundary_term(const float *P_c, int i, int j, i
                       : (order == 4 ? boundary_term_n<4>(P_c, i, j, k, Ng, S) : boundary_term_n<6>(P_c, i, j, k, Ng, S));
 }
 
+// Quotient and remainder of v / n for 0 <= v < n^3 < 2^31, from a reciprocal.  The conversion of v,
+// the reciprocal (2 ulp) and the product are off by less than 2^-21.4 together, of a quotient
+// below 2^20.7: less than one, so one step of correction on the exact integer remainder is enough.
+// (Each particle kernel decodes its lattice site with two of these; with integer divisions, and a
+// clearing pass in the atomic deposit: 21 evaluations of 64 boxes of 48^3 particles 16.90 ms, now
+// 16.67; one force evaluation on 64 boxes of 96^3 cells 826 us, now 816.)
+__device__ __forceinline__ int div_small(int v, int n, float inv, int &rem) {
+    int q = __float2int_rz((float)v * inv);
+    rem = v - q * n;
+    if (rem >= n) {
+        rem -= n;
+        ++q;
+    } else if (rem < 0) {
+        rem += n;
+        --q;
+    }
+    return q;
+}
+
 __device__ __forceinline__ void decode_local(int local, int n, int &i, int &j, int &k) {
-    k = local % n;
-    const int t = local / n;
-    j = t % n;
-    i = t / n;
+    const float inv = __fdividef(1.0f, (float)n);
+    i = div_small(div_small(local, n, inv, k), n, inv, j);
 }
 
 // Blocks of 256 lattice sites for the kernels that gather from the mesh: 4 x (64 / z) x z sites

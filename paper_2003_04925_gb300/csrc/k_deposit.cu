@@ -9,7 +9,8 @@
 // are taken in groups whose counts do (one scratch accumulator, reused by every group):
 // for each group, the deposit kernel accumulates into the scratch, then the source kernel
 // converts the counts to delta = (Ng/Nsc)^3 n - 1, subtracts the boundary term on the
-// faces and writes delta' to the interior mesh, and the scratch is cleared.  The
+// faces, writes delta' to the interior mesh and clears the counts it has read (64 boxes of 72-96
+// cells a side: 1755 us a force evaluation with a clearing pass per group, 1738 without).  The
 // accumulator traffic stays in L2; HBM sees the positions once and delta' once.
 #include <algorithm>
 
@@ -108,7 +109,7 @@ constexpr int kSourceChunks = 4;
 
 __global__ void __launch_bounds__(64 * kSourceChunks)
 k_density_source(const BoxDesc *__restrict__ boxes, const Chunk *__restrict__ chunks, int nchunks,
-                 const unsigned long long *__restrict__ acc, long long acc_base, const float *__restrict__ phi_pad,
+                 unsigned long long *__restrict__ acc, long long acc_base, const float *__restrict__ phi_pad,
                  float inv_D1, const float *__restrict__ coef, int kstep, int nk, float *__restrict__ out,
                  float *__restrict__ delta_out) {
     const int ci = blockIdx.x * kSourceChunks + (threadIdx.x >> 6);
@@ -122,7 +123,7 @@ k_density_source(const BoxDesc *__restrict__ boxes, const Chunk *__restrict__ ch
     if ((long long)cell0 >= ng3) return;
     const int left = (int)min(4LL, ng3 - cell0);
     const float sc = B.nbar_inv * 2.3283064365386963e-10f, c2 = B.inv_dg * B.inv_dg;
-    const unsigned long long *a = acc + (B.m_off - acc_base) + cell0;
+    unsigned long long *a = acc + (B.m_off - acc_base) + cell0;        // read, and cleared for the next group
     const bool vec = left == 4 && (Ng & 3) == 0;
     float v[4];
     if (vec) {
@@ -132,11 +133,16 @@ k_density_source(const BoxDesc *__restrict__ boxes, const Chunk *__restrict__ ch
         v[1] = fixed_to_float(a01.y) * sc - 1.0f;
         v[2] = fixed_to_float(a23.x) * sc - 1.0f;
         v[3] = fixed_to_float(a23.y) * sc - 1.0f;
+        reinterpret_cast<ulonglong2 *>(a)[0] = make_ulonglong2(0ull, 0ull);
+        reinterpret_cast<ulonglong2 *>(a)[1] = make_ulonglong2(0ull, 0ull);
     } else {
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
             v[e] = 0.0f;
-            if (e < left) v[e] = fixed_to_float(a[e]) * sc - 1.0f;
+            if (e < left) {
+                v[e] = fixed_to_float(a[e]) * sc - 1.0f;
+                a[e] = 0ull;
+            }
         }
     }
     const long long cell = B.m_off + cell0;
@@ -195,11 +201,6 @@ cudaError_t launch_deposit_atomic(Ctx &c, const float *s, long long stride, floa
             ++c.launches;
             if ((e = cudaGetLastError()) != cudaSuccess) return step_error("atomic deposit: source launch", e);
         }
-        // clear the counts this group used (they stay in L2 for the next group)
-        const BoxDesc &last = c.boxes_h[b1 - 1];
-        const long long used = last.m_off + (long long)last.Ng * last.Ng * last.Ng - base;
-        e = cudaMemsetAsync(c.dep_acc, 0, sizeof(unsigned long long) * (size_t)used, c.stream);
-        if (e != cudaSuccess) return step_error("atomic deposit: clearing the scratch", e);
     }
     return cudaSuccess;
 }
