@@ -47,8 +47,8 @@ def parse():
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--dst", default="auto", choices=["auto", "tc", "tc4", "tc3", "simt", "radix"],
                     help="Poisson-solve form: the library's autotuner (auto, default: the fastest of the "
-                         "tensor-core forms and FP32 CUDA cores), tensor-core 3xTF32 in six passes (tc), "
-                         "4xTF32 (tc4), three passes (tc3: 3xTF32 z passes, 3xFP16 plane pass), dense FP32 CUDA cores (simt) or radix "
+                         "tensor-core forms and FP32 CUDA cores), tensor-core 3xTF32 in one-axis passes (tc), "
+                         "4xTF32 (tc4), three passes (tc3: 3xFP16 plane passes, elimination along x), dense FP32 CUDA cores (simt) or radix "
                          "(Bluestein) FP32 transforms (radix)")
     ap.add_argument("--forward-only", action="store_true",
                     help="only W + K forward runs of the batched form (for ncu launch lists)")
@@ -403,10 +403,11 @@ def study_cost(sc, torch, kw, W, steps, peaks):
 def kernel_roofline(kt, kw, clocks, peaks, form, box_frac=1.0):
     """Algorithmic bytes or flops per launch of each kernel class and the dominant one.
 
-    FP32 form: the five DST passes are dense products on CUDA cores (ALU bound,
-    2 Ng flops per cell per transform; pass 3 does two transforms).  Tensor-core
-    and radix forms: six passes (or three), each streaming its mesh once (HBM bound:
-    4 B read + 4 B written per cell).  Deposit: the positions once (12 B per particle) and the
+    FP32 form: dense products on CUDA cores (ALU bound, 2 Ng flops per cell per transform):
+    five passes, pass 3 with two transforms, or where passes 4 and 5 are empty, two plane
+    passes of two transforms around the elimination along x (HBM bound).  Tensor-core and
+    radix forms: three, five or six passes, each streaming its mesh once (HBM bound: 4 B read
+    + 4 B written per cell).  Deposit: the positions once (12 B per particle) and the
     Poisson source written once (4 B per cell).
     """
     nsc, ng = box_sizes(kw)
@@ -418,8 +419,10 @@ def kernel_roofline(kt, kw, clocks, peaks, form, box_frac=1.0):
     work = {"deposit": ("hbm", 12.0 * P + 4.0 * M),
             "kick_drift": ("hbm", 72.0 * P + 4.0 * MP)}
     if form == "tc3":
-        # three mesh passes: z forward, the plane pass (y, x forward, division, x, y inverse),
-        # z inverse; each streams the mesh once
+        # three mesh passes, each streaming the mesh once.  At FDA order 2 these are the forward
+        # plane pass (z and y), the elimination along x and the inverse plane pass; at orders 4
+        # and 6 (the names) z forward, the plane pass (y, x forward, division, x, y inverse) and
+        # z inverse
         names = ["dst_1_z_fwd", "dst_2_plane", "dst_3_z_inv", None, None, None]
         for nm in names[:3]:
             work[nm] = ("hbm", 8.0 * M)
@@ -428,8 +431,14 @@ def kernel_roofline(kt, kw, clocks, peaks, form, box_frac=1.0):
         # streaming its mesh once
         names = ["dst_1_z_fwd", "dst_2_y_fwd", "dst_3_x_fwd_div", "dst_4_z_inv", "dst_5_y_inv",
                  "dst_6_x_inv"]
-        for i, nm in enumerate(names):
-            work[nm] = ("hbm", 8.0 * M)
+        if form != "radix" and kt["dst_6"] < 0.5 * kt["dst_1"]:
+            names = names[:2] + ["dst_3_x_elimination"] + names[3:5] + [None]
+        for nm in names:
+            if nm:
+                work[nm] = ("hbm", 8.0 * M)
+    elif kt["dst_4"] < 0.5 * kt["dst_1"]:
+        names = ["dst_1_plane_fwd", "dst_2_x_elimination", "dst_3_plane_inv", None, None, None]
+        work.update({names[0]: ("alu", 2 * dense), names[1]: ("hbm", 8.0 * M), names[2]: ("alu", 2 * dense)})
     else:
         names = ["dst_1_z_fwd", "dst_2_y_fwd", "dst_3_x_solve", "dst_4_y_inv", "dst_5_z_inv", None]
         for i, nm in enumerate(names):
@@ -682,8 +691,8 @@ def run_gpu(args, rank, world, local_rank):
                     "particle_steps_per_step": work,
                     "l2": "working set %.2f GB > 129 MB L2, no flush" % (ws_bytes / 1e9),
                     "parallelism": "boxes split over %d GPU(s)" % world,
-                    "dst": {"tc": "tcgen05 3xTF32, six passes", "tc4": "tcgen05 4xTF32, six passes",
-                            "tc3": "tcgen05 three passes (3xTF32 z, 3xFP16 planes)", "simt": "FP32 CUDA cores",
+                    "dst": {"tc": "tcgen05 3xTF32, one-axis passes", "tc4": "tcgen05 4xTF32, one-axis passes",
+                            "tc3": "tcgen05 three passes (3xFP16 planes, elimination along x)", "simt": "FP32 CUDA cores",
                             "radix": "FP32 CUDA cores, radix (Bluestein) transforms"}[args.dst]}),
                 "gpu_launches": int(launches * args.steps), "clocks": clk,
                 "roofline": roofline, "cpu_baseline": cpu, "e2e": e2e}
@@ -719,11 +728,11 @@ def deposit_choice(sc, st):
 def dst_choice(sc, st):
     """The Poisson-solve form in use and, under the autotuner, the candidates it timed (ms per
     solve of all boxes; both forms meet the accuracy bound)."""
-    names = {sc.SCOLA_DST_TC_3XTF32: "tensor cores, 3xTF32, six passes", sc.SCOLA_DST_TC_4XTF32: "tensor cores, 4xTF32",
-             sc.SCOLA_DST_TC_3PASS: "tensor cores, three passes (3xTF32 z, 3xFP16 planes)", sc.SCOLA_DST_SIMT: "FP32 CUDA cores",
+    names = {sc.SCOLA_DST_TC_3XTF32: "tensor cores, 3xTF32, one-axis passes", sc.SCOLA_DST_TC_4XTF32: "tensor cores, 4xTF32",
+             sc.SCOLA_DST_TC_3PASS: "tensor cores, three passes (3xFP16 planes, elimination along x)", sc.SCOLA_DST_SIMT: "FP32 CUDA cores",
              sc.SCOLA_DST_RADIX: "FP32 CUDA cores, radix (Bluestein) transforms"}
     cand = st["ms_dst_candidates"]
-    order = ("tensor cores, 3xTF32, six passes", "FP32 CUDA cores", "tensor cores, three passes (3xTF32 z, 3xFP16 planes)",
+    order = ("tensor cores, 3xTF32, one-axis passes", "FP32 CUDA cores", "tensor cores, three passes (3xFP16 planes, elimination along x)",
              "FP32 CUDA cores, radix (Bluestein) transforms")
     return {"kept": names.get(st["dst_form"], "not chosen"),
             "candidates_ms": {n: round(t, 4) for n, t in zip(order, cand) if t > 0}}

@@ -78,7 +78,7 @@ typedef enum scola_dst_variant {
                                     where every Ng allows it), the dense FP32 form and the radix
                                     form, timed once on the context's boxes before the first
                                     evolution (where Ng > 222 excludes the dense FP32 form: the
-                                    six-pass tensor-core form alone; where Ng > 240 excludes the
+                                    one-axis tensor-core form alone; where Ng > 240 excludes the
                                     tensor cores: the radix form) */
 } scola_dst_variant;
 
@@ -233,7 +233,7 @@ typedef struct scola_stats {
                                      the requested one, or the autotuner's pick under AUTO
                                      (0 until the first scola_forward / scola_setup_boxes) */
     double ms_dst_candidates[4];  /* AUTO: autotuner timings of one Poisson solve: tensor cores
-                                     in six passes, dense FP32, tensor cores in three passes,
+                                     one axis per pass, dense FP32, tensor cores in three passes,
                                      radix FP32; 0 = not timed */
     int32_t adjoint_potentials_kept; /* 1: with checkpoints at every force evaluation the
                                      forward run also keeps each evaluation's padded potential

@@ -1,7 +1,8 @@
 // Dirichlet Poisson solve on the 5th-generation tensor cores (App. C, Eqs. 62-71).
 //
-// The 3D DST-I is applied as six dense pencil products over rows whose transform
-// axis is contiguous in memory.  For a tile of 256 such rows X (256 x Ng) a pass
+// The 3D DST-I is applied as dense pencil products over rows whose transform axis is
+// contiguous in memory: six at FDA orders 4 and 6, four around the elimination along x at
+// order 2 (P_M, P_MI below).  For a tile of 256 such rows X (256 x Ng) a pass
 // computes D^T = S X^T on the tensor cores (S_kn = sin(pi (k+1)(n+1)/(Ng+1)),
 // symmetric): the sine matrix is the M = 128 operand (rows n < Ng, resident in
 // shared memory for the whole launch) and the data rows are the N = 256 operand, so
@@ -10,7 +11,7 @@
 // writes contiguous runs of out[n][row]: every pass stores its result transposed,
 // out[col][row], so that the next pass again finds its axis contiguous:
 //
-//   pass  input rows (axis)    k    writes              epilogue
+//   pass  input rows (axis)    k    writes              epilogue   (orders 4 and 6)
 //   z+    src[i][j][k]  (i,j)  k    W1[n][i][j]         (src: delta' from the deposit)
 //   y+    W1[n][i][j]   (n,i)  j    W2[m][n][i]
 //   x+    W2[m][n][i]   (m,n)  i    W3[l][m][n]         / (lambda_l + lambda_m + lambda_n)

@@ -8,7 +8,9 @@
 //  deposit       B^sCOLA (Sec. 3.4.1) and the boundary source delta' = delta -
 //                Lap Phi_BCs (Eq. 62), by brick binning: k_deposit.cu.
 //  pad           ghost layers of the potential <- D1(a_K) * shell (LEP, Eq. 23).
-//  poisson       the zero-boundary solve of App. C on delta': dense DST-I along z,
+//  poisson       the zero-boundary solve of App. C on delta' (here the dense FP32 form
+//                for orders 4 and 6 and for Ng > 128; order 2 up to 128: k_dst_small.cu and
+//                k_dst_tri.cu): dense DST-I along z,
 //                along y, then along x with the division
 //                by lambda_l + lambda_m + lambda_n (Eq. 71) and the inverse x
 //                transform, then inverse y, then inverse z with the 8/(Ng+1)^3
