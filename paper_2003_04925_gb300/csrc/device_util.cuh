@@ -128,11 +128,11 @@ __device__ __forceinline__ void decode_local(int local, int n, int &i, int &j, i
 // Boxes that blocks would cover with more than an eighth of idle lanes (25 sites a side: 83 %)
 // keep the runs: block_z = 0.
 __host__ __device__ inline int block_tiles(int Nsc, int bz) {
-    const int by = 64 / bz;
-    return ((Nsc + 3) / 4) * ((Nsc + by - 1) / by) * ((Nsc + bz - 1) / bz);
+    const int sy = bz == 16 ? 2 : 3, sz = bz == 16 ? 4 : 3;
+    return ((Nsc + 3) >> 2) * ((Nsc + (1 << sy) - 1) >> sy) * ((Nsc + bz - 1) >> sz);
 }
 __host__ __device__ inline int block_z(int Nsc) {
-    const int bz = Nsc % 16 == 0 ? 16 : 8;
+    const int bz = (Nsc & 15) == 0 ? 16 : 8;
     return 8LL * 256 * block_tiles(Nsc, bz) <= 9LL * Nsc * Nsc * Nsc ? bz : 0;
 }
 __host__ __device__ inline int block_count(int Nsc) {
@@ -143,19 +143,16 @@ __host__ __device__ inline int block_count(int Nsc) {
 __device__ __forceinline__ bool block_site(int q, int t, int Nsc, int &i, int &j, int &k) {
     const int bz = block_z(Nsc);
     if (bz == 0) {
-        const int local = q * 256 + t;
-        k = local % Nsc;
-        const int r = local / Nsc;
-        j = r % Nsc;
-        i = r / Nsc;
+        decode_local(q * 256 + t, Nsc, i, j, k);
         return i < Nsc;
     }
-    const int by = 64 / bz;
-    const int nz = (Nsc + bz - 1) / bz, ny = (Nsc + by - 1) / by;
-    const int r = q / nz;
-    k = (q - r * nz) * bz + (t & (bz - 1));
-    j = (r % ny) * by + ((t & 63) / bz);
-    i = (r / ny) * 4 + (t >> 6);
+    const int sy = bz == 16 ? 2 : 3, sz = bz == 16 ? 4 : 3;
+    const int nz = (Nsc + bz - 1) >> sz, ny = (Nsc + (1 << sy) - 1) >> sy;
+    int bj, bk;
+    const int r = div_small(q, nz, __fdividef(1.0f, (float)nz), bk);
+    i = (div_small(r, ny, __fdividef(1.0f, (float)ny), bj) << 2) + (t >> 6);
+    j = (bj << sy) + ((t & 63) >> sz);
+    k = (bk << sz) + (t & (bz - 1));
     return i < Nsc && j < Nsc && k < Nsc;
 }
 
