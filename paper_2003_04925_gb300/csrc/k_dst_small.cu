@@ -123,7 +123,7 @@ cudaError_t init_small_kernels() {
 }
 
 // The dense FP32 form takes the plane passes where every mesh fits and the order is 2.
-bool small_supported(const Ctx &c) { return c.prm.fda_order == 2 && c.max_ng <= kSmallMaxN && c.max_ng >= 2; }
+bool small_supported(const Ctx &c) { return c.prm.fda_order == 2 && c.max_ng <= kSmallMaxN; }
 
 cudaError_t launch_small_pass(Ctx &c, int pass, const float *in, float *w1, float *out_pad) {
     switch (pass) {

@@ -133,10 +133,9 @@ __global__ void __launch_bounds__(2 * kTriW * kTriParts) k_dst_tri(const __grid_
         float *mt = meet + (int)((q - lo) & 1) * 2 * parts * kTriW;
         mt[side * kTriW] = y;
         __syncthreads();
-        if (mine) {
-            const float ca = cs[(half - 1) * kTriW], cb = cs[(Ng - half - 1) * kTriW];
-            const float ua = fmaf(ca, mt[kTriW], mt[0]) * *inv;
-            float u = side ? fmaf(cb, ua, mt[kTriW]) : ua;
+        if (mine && n > 0) {                                // (a mesh of one cell has no second half)
+            const float ua = fmaf(cs[(half - 1) * kTriW], mt[kTriW], mt[0]) * *inv;
+            float u = side ? fmaf(cs[(n - 1) * kTriW], ua, mt[kTriW]) : ua;     // (row b = n - 1 there)
             mine[(n - 1) * step] = u;
             for (int k0 = n - 2; k0 >= 0; k0 -= kTriB) {
                 float cv[kTriB], yv[kTriB];
