@@ -213,8 +213,9 @@ typedef struct scola_stats {
     double ms_lpt;                /* initial-condition and 2LPT stage, device time (on the
                                      first call, plus the deposit autotuner's runs) */
     double ms_evolve;             /* gather + evolution + scatter, device time */
-    int64_t kernel_launches;      /* kernels launched by the last forward call (a full-box Fourier
-                                     transform of the initial conditions counts one per axis) */
+    int64_t kernel_launches;      /* kernels launched by the last forward call: the library's own
+                                     (scola_own_kernel_launches) and those of its full-box
+                                     Fourier transforms (cuFFT), as captured from their plans */
     int32_t deposit_form;         /* the form in use: SCOLA_DEPOSIT_SORTED or _ATOMIC (0 before
                                      the first scola_forward / scola_setup_boxes) */
     int32_t deposit_threads;      /* threads per brick CTA of the sorted form, else 0 */
@@ -634,6 +635,9 @@ scola_status scola_generate_white_noise(scola_ctx *ctx, uint64_t seed, float *w_
 scola_status scola_tcola(scola_ctx *ctx, const float *w_dev, float *x_dev, float *p_dev);
 
 scola_status scola_get_stats(const scola_ctx *ctx, scola_stats *out);
+/* Kernels of this library alone, without cuFFT's, launched by the last scola_forward or
+ * scola_tcola call (0 before the first, and for a NULL context). */
+int64_t scola_own_kernel_launches(const scola_ctx *ctx);
 const char *scola_status_string(scola_status status);
 const char *scola_last_error(void);
 

@@ -90,6 +90,7 @@ _sig = {
                                        _P(c_int64)]),
     "scola_time_table": (c_int32, [_P(ScolaParams)] + [c_void_p] * 7),
     "scola_get_stats": (c_int32, [c_void_p, _P(ScolaStats)]),
+    "scola_own_kernel_launches": (c_int64, [c_void_p]),
     "scola_set_profiling": (c_int32, [c_void_p, c_int32]),
     "scola_kernel_times": (c_int32, [c_void_p, _P(c_double), c_int32]),
     "scola_tcola_kernel_times": (c_int32, [c_void_p, _P(c_double), c_int32]),
@@ -287,6 +288,7 @@ def scola_get_stats(ctx):
     out = {name: getattr(st, name) for name, _ in ScolaStats._fields_}
     out["ms_deposit_candidates"] = list(out["ms_deposit_candidates"])
     out["ms_dst_candidates"] = list(out["ms_dst_candidates"])
+    out["own_kernel_launches"] = _lib.scola_own_kernel_launches(ctx)
     return out
 
 

@@ -41,7 +41,7 @@ struct BoxGeom {                         // one box of the tiling: Np,sCOLA, Ng,
 
 struct StageGraph {                      // a full-box stage's launches as a graph (run_graphed)
     cudaGraphExec_t exec = nullptr;
-    long long kernels = 0;
+    long long kernels = 0, fft_kernels = 0;
     int runs = 0;
     bool refused = false;
 };
@@ -54,6 +54,9 @@ struct scola_ctx : public Ctx {
     std::vector<BoxGeom> ctx_geo;        // the context's boxes
     cudaStream_t cap_stream = nullptr;   // stream used only to capture the evolution graph
     long long graph_kernels = 0;         // kernels in the evolution graph
+    int r2c_kernels = 0, c2r_kernels = 0;  // cuFFT kernels of one full-box transform
+    long long fft_launches = 0;          // cuFFT kernels so far (Ctx::launches: this library's own)
+    long long own_kernels = 0;           // own kernels of the last scola_forward or scola_tcola
     float *w_h2d = nullptr, *x_h2d = nullptr, *p_h2d = nullptr;  // buffers of scola_forward_host
     bool profiling = false;
     std::vector<cudaEvent_t> prof_ev;    // KC_COUNT + 1 events per force evaluation
@@ -81,11 +84,11 @@ struct scola_ctx : public Ctx {
         }                                                                            \
     } while (0)
 
-// A full-box transform of the LPT stage, counted as one kernel per axis.
-#define CT(call)                                                                     \
+// A full-box transform of the LPT stage and the cuFFT kernels it launches.
+#define CT(call, kernels)                                                            \
     do {                                                                             \
         CF(call);                                                                    \
-        c->launches += 3;                                                            \
+        c->fft_launches += (kernels);                                                \
     } while (0)
 
 #define CS(call)                                                                     \
@@ -630,6 +633,33 @@ scola_status tcola_alloc(scola_ctx *c) {
     return SCOLA_OK;
 }
 
+// Kernels that one execution of a cuFFT plan launches, from a capture that is not run (0 where the
+// capture is refused).
+template <typename Exec>
+int captured_kernels(scola_ctx *c, cufftHandle plan, Exec exec) {
+    size_t n = 0;
+    int kernels = 0;
+    cudaGraph_t graph = nullptr;
+    if (cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
+    const bool ran = cufftSetStream(plan, c->cap_stream) == CUFFT_SUCCESS && exec() == CUFFT_SUCCESS;
+    const bool ended = cudaStreamEndCapture(c->cap_stream, &graph) == cudaSuccess;
+    if (ran && ended && cudaGraphGetNodes(graph, nullptr, &n) == cudaSuccess) {
+        std::vector<cudaGraphNode_t> nodes(n);
+        if (n && cudaGraphGetNodes(graph, nodes.data(), &n) == cudaSuccess)
+            for (cudaGraphNode_t node : nodes) {
+                cudaGraphNodeType type;
+                if (cudaGraphNodeGetType(node, &type) == cudaSuccess && type == cudaGraphNodeTypeKernel) ++kernels;
+            }
+    }
+    if (graph) cudaGraphDestroy(graph);
+    cufftSetStream(plan, c->stream);
+    cudaGetLastError();
+    return kernels;
+}
+
 scola_status build(scola_ctx *c, const std::vector<BoxGeom> &all_geo) {
     const scola_params &p = c->prm;
     // the boxes this context evolves: all, or the range [box_first, box_first + box_count)
@@ -1000,6 +1030,8 @@ scola_status build(scola_ctx *c, const std::vector<BoxGeom> &all_geo) {
     for (int i = 0; i < 4; ++i) CK(cudaEventCreate(&c->ev[i]));
     for (int i = 0; i < 2; ++i) CK(cudaEventCreate(&c->tc_ev[i]));
     CK(cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking));
+    c->r2c_kernels = captured_kernels(c, c->plan_r2c, [&]() { return cufftExecR2C(c->plan_r2c, c->g[0], c->ck); });
+    c->c2r_kernels = captured_kernels(c, c->plan_c2r, [&]() { return cufftExecC2R(c->plan_c2r, c->ct, c->g[0]); });
 
     c->stats.nboxes = count;
     c->stats.box_particles = c->P_all;
@@ -1026,7 +1058,7 @@ scola_status run_graphed(scola_ctx *c, StageGraph &G, Body body) {
     if (G.runs++ == 0 || G.refused || cap != cudaStreamCaptureStatusNone) return body();
     if (!G.exec) {
         const cudaStream_t user = c->stream;
-        const long long before = c->launches;
+        const long long before = c->launches, fft_before = c->fft_launches;
         cudaGraph_t graph = nullptr;
         CK(cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal));
         c->stream = c->cap_stream;
@@ -1040,7 +1072,9 @@ scola_status run_graphed(scola_ctx *c, StageGraph &G, Body body) {
         if (st == SCOLA_OK && e == cudaSuccess) e = cudaGraphInstantiate(&G.exec, graph, 0);
         if (graph) cudaGraphDestroy(graph);
         G.kernels = c->launches - before;
+        G.fft_kernels = c->fft_launches - fft_before;
         c->launches = before;
+        c->fft_launches = fft_before;
         if (st != SCOLA_OK || e != cudaSuccess) {              // keep launching one by one
             cudaGetLastError();
             G.exec = nullptr;
@@ -1050,18 +1084,19 @@ scola_status run_graphed(scola_ctx *c, StageGraph &G, Body body) {
     }
     CK(cudaGraphLaunch(G.exec, c->stream));
     c->launches += G.kernels;
+    c->fft_launches += G.fft_kernels;
     return SCOLA_OK;
 }
 
 // A.1-A.2 on the full box into the context's grids.
 scola_status lpt_stage(scola_ctx *c, const float *w) {
     const float invN3 = (float)(1.0 / (double)c->N3);
-    CT(cufftExecR2C(c->plan_r2c, const_cast<cufftReal *>(reinterpret_cast<const cufftReal *>(w)), c->ck));
+    CT(cufftExecR2C(c->plan_r2c, const_cast<cufftReal *>(reinterpret_cast<const cufftReal *>(w)), c->ck), c->r2c_kernels);
     CK(launch_colour(*c, c->ck));
     const size_t cbytes = sizeof(cufftComplex) * (size_t)c->Np * c->Np * (c->Np / 2 + 1);
     CK(launch_inv_laplacian(*c, c->ck, c->cp, 1.0f));
     CK(cudaMemcpyAsync(c->ct, c->cp, cbytes, cudaMemcpyDeviceToDevice, c->stream));
-    CT(cufftExecC2R(c->plan_c2r, c->ct, c->phi1));
+    CT(cufftExecC2R(c->plan_c2r, c->ct, c->phi1), c->c2r_kernels);
     CK(launch_gradient(*c, c->phi1, c->psi1));
     if (c->prm.lpt_order == 1) {
         // Zel'dovich frame: no second-order potential or displacements
@@ -1071,18 +1106,18 @@ scola_status lpt_stage(scola_ctx *c, const float *w) {
     }
     for (int a = 0; a < 3; ++a) {
         CK(launch_second_derivative(*c, c->cp, c->ct, a, a));
-        CT(cufftExecC2R(c->plan_c2r, c->ct, c->g[a]));
+        CT(cufftExecC2R(c->plan_c2r, c->ct, c->g[a]), c->c2r_kernels);
     }
     CK(launch_source_init(*c, c->g[0], c->g[1], c->g[2], c->g[3]));
     const int pairs[3][2] = {{0, 1}, {0, 2}, {1, 2}};
     for (auto &pr : pairs) {
         CK(launch_second_derivative(*c, c->cp, c->ct, pr[0], pr[1]));
-        CT(cufftExecC2R(c->plan_c2r, c->ct, c->g[0]));
+        CT(cufftExecC2R(c->plan_c2r, c->ct, c->g[0]), c->c2r_kernels);
         CK(launch_source_sub(*c, c->g[0], c->g[3]));
     }
-    CT(cufftExecR2C(c->plan_r2c, c->g[3], c->ct));
+    CT(cufftExecR2C(c->plan_r2c, c->g[3], c->ct), c->r2c_kernels);
     CK(launch_inv_laplacian(*c, c->ct, c->ct, invN3));
-    CT(cufftExecC2R(c->plan_c2r, c->ct, c->phi2));
+    CT(cufftExecC2R(c->plan_c2r, c->ct, c->phi2), c->c2r_kernels);
     CK(launch_gradient(*c, c->phi2, c->psi2));
     return SCOLA_OK;
 }
@@ -1102,7 +1137,7 @@ scola_status run_lpt(scola_ctx *c, const float *w, float *delta_out) {
     if (delta_out) {
         const size_t cbytes = sizeof(cufftComplex) * (size_t)c->Np * c->Np * (c->Np / 2 + 1);
         CK(cudaMemcpyAsync(c->ct, c->ck, cbytes, cudaMemcpyDeviceToDevice, c->stream));
-        CT(cufftExecC2R(c->plan_c2r, c->ct, delta_out));
+        CT(cufftExecC2R(c->plan_c2r, c->ct, delta_out), c->c2r_kernels);
     }
     return SCOLA_OK;
 }
@@ -1781,7 +1816,7 @@ scola_status scola_box_particle_ids(scola_ctx *c, int64_t *gid) {
 
 scola_status scola_forward(scola_ctx *c, const float *w, float *x, float *p) {
     if (!c || !w || !x || !p) return invalid("NULL argument");
-    const long long before = c->launches;
+    const long long before = c->launches, fft_before = c->fft_launches;
     long long graph_kernels = 0;
     CK(cudaEventRecord(c->ev[0], c->stream));
     CS(run_lpt(c, w, nullptr));
@@ -1803,7 +1838,8 @@ scola_status scola_forward(scola_ctx *c, const float *w, float *x, float *p) {
     CK(cudaEventRecord(c->ev[2], c->stream));
     c->setup_done = true;
     c->have_forward = true;
-    c->stats.kernel_launches = (c->launches - before) + graph_kernels;
+    c->own_kernels = (c->launches - before) + graph_kernels;
+    c->stats.kernel_launches = c->own_kernels + (c->fft_launches - fft_before);
     return SCOLA_OK;
 }
 
@@ -1819,13 +1855,14 @@ scola_status scola_tcola(scola_ctx *c, const float *w, float *x, float *p) {
         set_error("the periodic tCOLA run is built for FDA order 2");
         return SCOLA_ERR_UNSUPPORTED;
     }
-    const long long before = c->launches;
+    const long long before = c->launches, fft_before = c->fft_launches;
     c->have_forward = false;            // the adjoint's LPT spectra are replaced
     CS(run_lpt(c, w, nullptr));
     c->tc_timed = false;
     CS(run_tcola(c, false));
     CK(launch_tc_final(*c, x, p));
-    c->stats.kernel_launches = c->launches - before;
+    c->own_kernels = c->launches - before;
+    c->stats.kernel_launches = c->own_kernels + (c->fft_launches - fft_before);
     return SCOLA_OK;
 }
 
@@ -2245,6 +2282,8 @@ scola_status scola_power_spectrum(scola_ctx *c, const float *delta, int32_t nbin
     }
     return SCOLA_OK;
 }
+
+int64_t scola_own_kernel_launches(const scola_ctx *c) { return c ? c->own_kernels : 0; }
 
 scola_status scola_get_stats(const scola_ctx *cc, scola_stats *out) {
     if (!cc || !out) return invalid("NULL argument");
