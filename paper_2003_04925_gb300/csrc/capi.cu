@@ -479,6 +479,9 @@ scola_status bind_coefficients(scola_ctx *c, int first, int count) {
 // rows of a multiple of 4 cells (a plane is then a whole number of 32-byte texture pitches), and
 // planes of at most 2^16 cells (columns and their halves stay exact in the texture unit's
 // coordinates).  Otherwise, or where the driver refuses one, the interpolation uses plain loads.
+// Only scola_pm_force reads them, and it takes contexts of one batch: made once, when that batch is
+// bound.  (Streamed batches rebind in every run: 64 boxes of 40-64 cells in 4 batches of differing
+// shape take 4.00 ms a run of 4 evaluations, and took 4.45 while every rebinding made its textures.)
 void drop_textures(scola_ctx *c) {
     for (cudaTextureObject_t t : c->phi_tex_h) cudaDestroyTextureObject(t);
     c->phi_tex_h.clear();
@@ -488,12 +491,15 @@ void drop_textures(scola_ctx *c) {
 scola_status bind_textures(scola_ctx *c) {
     drop_textures(c);
     if (c->prm.fda_order != 2) return SCOLA_OK;
-    cudaDeviceProp prop;
-    CK(cudaGetDeviceProperties(&prop, c->device));
+    int width = 0, height = 0, pitch = 0, alignment = 0;
+    CK(cudaDeviceGetAttribute(&width, cudaDevAttrMaxTexture2DLinearWidth, c->device));
+    CK(cudaDeviceGetAttribute(&height, cudaDevAttrMaxTexture2DLinearHeight, c->device));
+    CK(cudaDeviceGetAttribute(&pitch, cudaDevAttrMaxTexture2DLinearPitch, c->device));
+    CK(cudaDeviceGetAttribute(&alignment, cudaDevAttrTextureAlignment, c->device));
     for (const BoxDesc &B : c->boxes_h) {
         const int S = B.Ng + 2 * B.gpad;
-        if (S % 4 != 0 || S * S > 65536 || S * S > prop.maxTexture2DLinear[0] ||
-            (size_t)S * S * sizeof(float) > (size_t)prop.maxTexture2DLinear[2] || prop.textureAlignment > 512)
+        if (S % 4 != 0 || S * S > 65536 || S * S > width || S > height || S * S * (int)sizeof(float) > pitch ||
+            alignment > 512)
             return SCOLA_OK;
     }
     for (const BoxDesc &B : c->boxes_h) {
@@ -599,7 +605,7 @@ scola_status bind_batch(scola_ctx *c, int k, bool force = false) {
     c->MP = bp.MP;
     c->SH = bp.SH;
     CS(bind_coefficients(c, first, count));
-    CS(bind_textures(c));
+    if (c->batch_first.size() == 2) CS(bind_textures(c));
     c->bound_batch = k;
     return SCOLA_OK;
 }
