@@ -322,6 +322,7 @@ void plan_batch(const scola_ctx *c, const std::vector<BoxGeom> &tiling_geo, int 
         B.q2u = (float)((double)g.ng / g.nsc);
         B.nbar_inv = (float)std::pow((double)g.ng / g.nsc, 3);
         B.dg_d = dg;
+        B.inv_2ng_d = 1.0 / (2.0 * g.ng);
         const int t3[3] = {B.tx, B.ty, B.tz};
         for (int a = 0; a < 3; ++a) B.origin_d[a] = ((double)t3[a] * ntile - g.nbuf) * c->dq;
         bp.boxes.push_back(B);

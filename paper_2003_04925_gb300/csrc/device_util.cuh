@@ -260,8 +260,8 @@ __device__ __forceinline__ void shell_stencil_r(const BoxDesc &B, const int pc[3
     }
 }
 
-// Unevaluated sums h + l of two floats (about 47 significant bits), for the C.3 shell: FP64 runs
-// at 1/64 of the FP32 rate on this GPU.  Sums by Knuth's two-sum, products by one FMA remainder
+// Unevaluated sums h + l of two floats (about 47 significant bits), for the C.3 shell where they
+// decide its rounding: FP64 runs at 1/64 of the FP32 rate on this GPU.  Sums by Knuth's two-sum, products by one FMA remainder
 // (Dekker 1971, Knuth TAOCP vol. 2, 4.2.2); the _rn intrinsics keep the compiler from fusing.
 struct FloatPair {
     float h, l;
@@ -282,6 +282,11 @@ __device__ __forceinline__ FloatPair pair_lerp(FloatPair a, FloatPair b, FloatPa
     r.l = __fadd_rn(r.l, __fadd_rn(a.l, tl));
     const float h = __fadd_rn(r.h, r.l);
     return {h, __fsub_rn(r.l, __fsub_rn(h, r.h))};
+}
+
+// Whether every value within e of x.h + x.l rounds to x.h (false for infinities and NaN).
+__device__ __forceinline__ bool pair_rounds(FloatPair x, float e) {
+    return __fadd_rn(x.h, __fadd_rn(x.l, e)) == x.h && __fadd_rn(x.h, __fsub_rn(x.l, e)) == x.h;
 }
 
 __device__ __forceinline__ int wrap(int v, int n) {

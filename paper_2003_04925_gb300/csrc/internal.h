@@ -45,6 +45,7 @@ struct BoxDesc {
     int gpad;                     // ghost layers per side of the padded potential: 2 N_ghost = FDA order
     int fda;                      // FDA order 2, 4, 6
     double dg_d, origin_d[3];     // FP64 box geometry (cell size, origin of the box frame)
+    double inv_2ng_d;             // 1 / (2 Ng) in FP64 (the C.3 shell stencil's offsets)
 };
 
 struct Chunk {                    // one CTA of a particle- or cell-parallel kernel

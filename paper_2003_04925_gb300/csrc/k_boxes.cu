@@ -7,10 +7,10 @@
 //  shell      C.3: phi1 trilinearly interpolated (periodic, nodes at (i+1/2) d)
 //             to the centre of every padded PM cell outside the interior; the
 //             stencil comes from exact integer arithmetic (shell_stencil_r), the
-//             seven linear interpolations run on pairs of floats (about 47 bits) and
-//             the result is rounded once to FP32 (LEP scaling by D1(a_K) happens per
-//             force evaluation, Eq. 23).  Runs once per run: 127 us for 64 boxes of
-//             96^3 cells, 561 us with FP64 products (bound by the FP64 pipe).
+//             result is the FP64 interpolation rounded once to FP32 (LEP scaling by
+//             D1(a_K) happens per force evaluation, Eq. 23): seven linear interpolations
+//             on pairs of floats, and where those leave the rounding open the eight
+//             products in FP64.  Runs once per run.
 //  scatter    B.2 and L+: tile particles only; x = (q + s) mod L and
 //             p = p_res + a^2 calH (-dD1/da Psi1 + dD2/da Psi2) at a_f (Eq. 55).
 //  box_ids    the global id of every box particle (integer, for inspection).
@@ -54,44 +54,97 @@ k_box_init(const BoxDesc *__restrict__ boxes, const Chunk *__restrict__ chunks,
     }
 }
 
-__global__ void __launch_bounds__(kChunk)
-k_shell(const BoxDesc *__restrict__ boxes, const Chunk *__restrict__ chunks,
-        const float *__restrict__ phi1, int N, int Ntile, float *__restrict__ shell) {
-    const Chunk ch = chunks[blockIdx.x];
-    const BoxDesc &B = boxes[ch.box];
-    const long long idx = (long long)ch.start + threadIdx.x;
-    if (idx >= shell_count(B.Ng, B.gpad)) return;
+// The eight phi1 values around shell cell `lane` of a chunk and the remainders of its offsets
+// rem / (2 Ng); the cell's place in the shells, or -1 beyond its box's.
+__device__ __forceinline__ long long shell_cell(const BoxDesc &B, const Chunk &ch, int lane, const float *__restrict__ phi1,
+                                                int N, int Ntile, float (&v)[2][2][2], int (&rem)[3]) {
+    const long long idx = (long long)ch.start + lane;
+    if (idx >= shell_count(B.Ng, B.gpad)) return -1;
     int pc[3];
     shell_coord(idx, B.Ng, B.gpad, pc[0], pc[1], pc[2]);
     int i0[3];
-    int rem[3];
     shell_stencil_r(B, pc, Ntile, i0, rem);
-    // the offsets r / (2 Ng) as float pairs: a quotient and its exact remainder over 2 Ng
-    const float den = 2.0f * (float)B.Ng, inv = 1.0f / den;
-    FloatPair f[3];
     // the two periodic node indices per axis (one modulo each)
     int ix[3][2];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-        const float r = (float)rem[a];
-        f[a].h = r * inv;
-        f[a].l = __fmaf_rn(-f[a].h, den, r) * inv;
         ix[a][0] = wrap(i0[a], N);
         ix[a][1] = ix[a][0] + 1 == N ? 0 : ix[a][0] + 1;
     }
     const long long NN = (long long)N * N;
-    FloatPair vx[2];
 #pragma unroll
-    for (int dx = 0; dx < 2; ++dx) {
-        FloatPair vy[2];
+    for (int dx = 0; dx < 2; ++dx)
 #pragma unroll
         for (int dy = 0; dy < 2; ++dy) {
             const float *row = phi1 + ix[0][dx] * NN + (long long)ix[1][dy] * N;
-            vy[dy] = pair_lerp({row[ix[2][0]], 0.0f}, {row[ix[2][1]], 0.0f}, f[2]);
+            v[dx][dy][0] = row[ix[2][0]], v[dx][dy][1] = row[ix[2][1]];
         }
-        vx[dx] = pair_lerp(vy[0], vy[1], f[1]);
+    return B.sh_off + idx;
+}
+
+// Every value is the FP64 sum of the eight products rounded once.  The interpolations between pairs
+// of floats decide that rounding in all but the cells where they come close to the middle of two
+// floats; those are gathered and computed in FP64 by the CTA's first lanes (offsets of a few bits, as
+// on meshes of two cells per particle, meet exact middles: one cell in 100).  64 boxes of 96^3 cells:
+// 147 us, 127 without the decision, 561 with FP64 everywhere (its pipe at 1/64 of the FP32 rate);
+// 303 with each thread finishing its own cell, 152 and 173 with 2 and 4 chunks of cells a CTA.
+__global__ void __launch_bounds__(kChunk, 8)
+k_shell(const BoxDesc *__restrict__ boxes, const Chunk *__restrict__ chunks, const float *__restrict__ phi1, int N,
+        int Ntile, float *__restrict__ shell) {
+    __shared__ int n_open;
+    __shared__ unsigned char open[kChunk];
+    const Chunk ch = chunks[blockIdx.x];
+    const BoxDesc &B = boxes[ch.box];
+    float v[2][2][2];
+    int rem[3];
+    if (threadIdx.x == 0) n_open = 0;
+    __syncthreads();
+    const long long own = shell_cell(B, ch, threadIdx.x, phi1, N, Ntile, v, rem);
+    if (own >= 0) {
+        // the offsets r / (2 Ng) as float pairs: a quotient and its exact remainder over 2 Ng
+        const float den = 2.0f * (float)B.Ng, inv = 1.0f / den;
+        FloatPair f[3], vx[2];
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            const float r = (float)rem[a];
+            f[a].h = r * inv;
+            f[a].l = __fmaf_rn(-f[a].h, den, r) * inv;
+        }
+        float top = 0.0f;
+#pragma unroll
+        for (int dx = 0; dx < 2; ++dx) {
+            FloatPair vy[2];
+#pragma unroll
+            for (int dy = 0; dy < 2; ++dy) {
+                top = fmaxf(top, fmaxf(fabsf(v[dx][dy][0]), fabsf(v[dx][dy][1])));
+                vy[dy] = pair_lerp({v[dx][dy][0], 0.0f}, {v[dx][dy][1], 0.0f}, f[2]);
+            }
+            vx[dx] = pair_lerp(vy[0], vy[1], f[1]);
+        }
+        const FloatPair r = pair_lerp(vx[0], vx[1], f[0]);
+        // An interpolation adds at most nine errors of 2^-46 of the largest corner (the offset's 2^-46
+        // of a difference of 2, and the roundings of the low parts), the three levels less than 2^-40
+        // of it; small corners (underflow), infinities and NaN are left open too.
+        if (top >= 0x1p-80f && pair_rounds(r, top * 0x1p-39f)) shell[own] = r.h;
+        else open[atomicAdd(&n_open, 1)] = (unsigned char)threadIdx.x;
     }
-    shell[B.sh_off + idx] = pair_lerp(vx[0], vx[1], f[0]).h;
+    __syncthreads();
+    for (int q = threadIdx.x; q < n_open; q += kChunk) {
+        const long long at = shell_cell(B, ch, open[q], phi1, N, Ntile, v, rem);
+        double g[3], sum = 0.0;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) g[a] = __dmul_rn((double)rem[a], B.inv_2ng_d);
+#pragma unroll
+        for (int dx = 0; dx < 2; ++dx)
+#pragma unroll
+            for (int dy = 0; dy < 2; ++dy) {
+                const double wxy = (dx ? g[0] : 1.0 - g[0]) * (dy ? g[1] : 1.0 - g[1]);
+#pragma unroll
+                for (int dz = 0; dz < 2; ++dz)
+                    sum = fma(wxy * (dz ? g[2] : 1.0 - g[2]), (double)v[dx][dy][dz], sum);
+            }
+        shell[at] = (float)sum;
+    }
 }
 
 __global__ void __launch_bounds__(kChunk)
