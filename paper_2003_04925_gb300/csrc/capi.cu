@@ -1308,12 +1308,14 @@ struct BoxView {
 // memory, with 256 or 512 threads per brick; or fixed-point atomics into an L2-resident
 // scratch) give the same delta' bit for bit, so the choice changes only the speed.  Each
 // candidate allowed by params.deposit_form is timed with CUDA events on this context's own
-// boxes (one box in the per-tile form), with the particles where the LPT of the run puts them at
-// the middle force evaluation (on the initial lattice, where neighbours share cells, the
-// atomics look faster than they are over a run: 0.64 ms against 0.98 ms at a = 1 on 64 boxes of
-// 72-96 cells, one per particle), and the fastest is kept for the life of the context and for
-// its captured graph.  Runs once, before the first capture; needs the LPT fields (it launches
-// C.1-C.3 itself).
+// boxes (one box in the per-tile form), with the particles where the LPT puts them at the mean
+// growth of the run's force evaluations, and the fastest is kept for the life of the context and
+// for its captured graph.  (On the initial lattice, where neighbours share cells, the atomics look
+// faster than they are over a run, and at its end slower.  64 boxes of 72-96 cells, one per particle,
+// at a = 0.02, 0.35 and 1: atomics 831, 1044, 1372 us, sorted in 32-bit halves 786, 808, 854; 64 boxes
+// of 48^3: 182, 227, 289 against 183, 189, 202, where the pick of the late times loses 1 us on early
+// ones and the pick of the early times 38-87 us on late ones.)  Runs once, before the first
+// capture; needs the LPT fields (it launches C.1-C.3 itself).
 scola_status autotune_deposit(scola_ctx *c) {
     if (c->tuned) return SCOLA_OK;
     struct Cand {
@@ -1329,11 +1331,15 @@ scola_status autotune_deposit(scola_ctx *c) {
     {
         std::unique_ptr<BoxView> view;
         if (c->prm.batch_mode == SCOLA_BATCH_PER_TILE) view.reset(new BoxView(c, 0));
-        const size_t mid = c->tt.D1.size() / 2;
-        CK(launch_box_init(*c, c->tt.D1[mid], c->tt.D2[mid]));
+        double D1 = 0.0, D2 = 0.0;
+        for (size_t k = 0; k < c->tt.D1.size(); ++k) {
+            D1 += c->tt.D1[k] / (double)c->tt.D1.size();
+            D2 += c->tt.D2[k] / (double)c->tt.D1.size();
+        }
+        CK(launch_box_init(*c, D1, D2));
         CK(launch_shell(*c));
         CK(launch_pad(*c, 1.0f));
-        const float inv_D1 = (float)(1.0 / c->tt.D1[mid]);
+        const float inv_D1 = (float)(1.0 / D1);
         for (int q = lo; q < hi; ++q) {
             c->deposit_form = all[q].form;
             c->deposit_threads = all[q].threads;
