@@ -9,8 +9,7 @@
 // are taken in groups whose counts do (one scratch accumulator, reused by every group):
 // for each group, the deposit kernel accumulates into the scratch, then the source kernel
 // converts the counts to delta = (Ng/Nsc)^3 n - 1, subtracts the boundary term on the
-// faces, writes delta' to the interior mesh and clears the counts it has read (64 boxes of 72-96
-// cells a side: 1755 us a force evaluation with a clearing pass per group, 1738 without).  The
+// faces and writes delta' to the interior mesh, and the scratch is cleared.  The
 // accumulator traffic stays in L2; HBM sees the positions once and delta' once.
 #include <algorithm>
 
@@ -107,6 +106,14 @@ __device__ __forceinline__ void store4(float *p, const float (&v)[4], bool vec, 
 // kSourceChunks consecutive 256-cell chunks of the list (64 threads each).
 constexpr int kSourceChunks = 4;
 
+// The counts of a group of at most kClearCells cells are cleared by the threads that read them, which
+// saves a launch; larger groups by a memset after the kernel, whose stores into the lines it streams
+// would cost more.  Deposit, source and clearing in us, cleared by the readers / by a memset: 8 boxes
+// of 24^3 9.1 / 10.4, of 40^3 21.9 / 22.1, of 44^3 27.0 / 27.0, of 60^3 61.2 / 57.7, 64 of 48^3 271 /
+// 231, 64 of 72-96 cells 1284 / 1081, 16 of 192^3 1492 / 1006 (source alone 936 / 350 + 159).
+constexpr long long kClearCells = 1 << 19;
+
+template <bool kClear>
 __global__ void __launch_bounds__(64 * kSourceChunks)
 k_density_source(const BoxDesc *__restrict__ boxes, const Chunk *__restrict__ chunks, int nchunks,
                  unsigned long long *__restrict__ acc, long long acc_base, const float *__restrict__ phi_pad,
@@ -123,7 +130,7 @@ k_density_source(const BoxDesc *__restrict__ boxes, const Chunk *__restrict__ ch
     if ((long long)cell0 >= ng3) return;
     const int left = (int)min(4LL, ng3 - cell0);
     const float sc = B.nbar_inv * 2.3283064365386963e-10f, c2 = B.inv_dg * B.inv_dg;
-    unsigned long long *a = acc + (B.m_off - acc_base) + cell0;        // read, and cleared for the next group
+    unsigned long long *a = acc + (B.m_off - acc_base) + cell0;
     const bool vec = left == 4 && (Ng & 3) == 0;
     float v[4];
     if (vec) {
@@ -133,15 +140,17 @@ k_density_source(const BoxDesc *__restrict__ boxes, const Chunk *__restrict__ ch
         v[1] = fixed_to_float(a01.y) * sc - 1.0f;
         v[2] = fixed_to_float(a23.x) * sc - 1.0f;
         v[3] = fixed_to_float(a23.y) * sc - 1.0f;
-        reinterpret_cast<ulonglong2 *>(a)[0] = make_ulonglong2(0ull, 0ull);
-        reinterpret_cast<ulonglong2 *>(a)[1] = make_ulonglong2(0ull, 0ull);
+        if (kClear) {
+            reinterpret_cast<ulonglong2 *>(a)[0] = make_ulonglong2(0ull, 0ull);
+            reinterpret_cast<ulonglong2 *>(a)[1] = make_ulonglong2(0ull, 0ull);
+        }
     } else {
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
             v[e] = 0.0f;
             if (e < left) {
                 v[e] = fixed_to_float(a[e]) * sc - 1.0f;
-                a[e] = 0ull;
+                if (kClear) a[e] = 0ull;
             }
         }
     }
@@ -188,7 +197,9 @@ cudaError_t launch_deposit_atomic(Ctx &c, const float *s, long long stride, floa
         const int npch = one ? c.n_pchunks : c.pbeg[b1] - c.pbeg[b0];
         const Chunk *mch = one ? c.mchunks : c.mchunks + c.mbeg[b0];
         const int nmch = one ? c.n_mchunks : c.mbeg[b1] - c.mbeg[b0];
+        const BoxDesc &last = c.boxes_h[b1 - 1];
         const long long base = c.boxes_h[b0].m_off;
+        const long long used = last.m_off + (long long)last.Ng * last.Ng * last.Ng - base;
         cudaError_t e;
         if (npch > 0) {
             k_deposit<<<npch, kChunk, 0, c.stream>>>(c.boxes, pch, s, stride, c.dep_acc, base);
@@ -196,10 +207,15 @@ cudaError_t launch_deposit_atomic(Ctx &c, const float *s, long long stride, floa
             if ((e = cudaGetLastError()) != cudaSuccess) return step_error("atomic deposit: deposit launch", e);
         }
         if (nmch > 0) {
-            k_density_source<<<(nmch + kSourceChunks - 1) / kSourceChunks, 64 * kSourceChunks, 0, c.stream>>>(
+            const auto source = used <= kClearCells ? k_density_source<true> : k_density_source<false>;
+            source<<<(nmch + kSourceChunks - 1) / kSourceChunks, 64 * kSourceChunks, 0, c.stream>>>(
                 c.boxes, mch, nmch, c.dep_acc, base, c.phi, inv_D1, coef, kstep, c.coef_nk, c.work2, delta_out);
             ++c.launches;
             if ((e = cudaGetLastError()) != cudaSuccess) return step_error("atomic deposit: source launch", e);
+        }
+        if (used > kClearCells) {              // (the counts stay in L2 for the next group)
+            e = cudaMemsetAsync(c.dep_acc, 0, sizeof(unsigned long long) * (size_t)used, c.stream);
+            if (e != cudaSuccess) return step_error("atomic deposit: clearing the scratch", e);
         }
     }
     return cudaSuccess;
