@@ -1911,8 +1911,9 @@ scola_status scola_set_checkpointing(scola_ctx *c, int32_t enable) {
         CS(dev_alloc(&c->lamPsi2, 3 * N3));
         CS(dev_alloc(&c->lam_phi1, N3));
         CS(dev_alloc(&c->lam_phi2, N3));
-        CS(dev_alloc(&c->d2, 6 * N3));
-        CS(dev_alloc(&c->lam_d2, 6 * N3));
+        c->d2_stride = (N3 + 3) / 4 * 4;
+        CS(dev_alloc(&c->d2, 6 * c->d2_stride));
+        CS(dev_alloc(&c->lam_d2, 6 * c->d2_stride));
     }
     return SCOLA_OK;
 }
@@ -2059,13 +2060,13 @@ scola_status lpt_adjoint(scola_ctx *c, float *lam_w) {
         CF(cufftExecC2R(c->plan_c2r, c->ct, c->g[0]));                // lam_S
         for (int q = 0; q < 6; ++q) {
             CK(launch_second_derivative(*c, c->cp, c->ct, pairs[q][0], pairs[q][1]));
-            CF(cufftExecC2R(c->plan_c2r, c->ct, c->d2 + (size_t)q * N3));
+            CF(cufftExecC2R(c->plan_c2r, c->ct, c->d2 + (size_t)q * c->d2_stride));
         }
         CK(launch_adj_source(*c, c->g[0], c->d2, c->lam_d2));
     }
     CF(cufftExecR2C(c->plan_r2c, c->lam_phi1, c->ck));
     for (int q = 0; second && q < 6; ++q) {
-        CF(cufftExecR2C(c->plan_r2c, c->lam_d2 + (size_t)q * N3, c->ct));
+        CF(cufftExecR2C(c->plan_r2c, c->lam_d2 + (size_t)q * c->d2_stride, c->ct));
         CK(launch_spec_d2_accumulate(*c, c->ct, c->ck, pairs[q][0], pairs[q][1]));
     }
     CK(launch_adj_colour(*c, c->ck, c->ct));

@@ -246,7 +246,11 @@ struct Ctx {
     float *adj = nullptr;                             // 12 x P backward particle state
     float *lamG = nullptr, *lam_phi_pad = nullptr, *adj_in = nullptr, *adj_out = nullptr;
     float *lam_shell = nullptr, *lamPsi1 = nullptr, *lamPsi2 = nullptr;
-    float *lam_phi1 = nullptr, *lam_phi2 = nullptr, *d2 = nullptr, *lam_d2 = nullptr;
+    float *lam_phi1 = nullptr, *lam_phi2 = nullptr;
+    // the six second derivatives and their adjoints, d2_stride = N3 rounded up to 4 floats apart
+    // (cuFFT takes real rows of 8-byte alignment, which an odd N3 alone would not keep)
+    float *d2 = nullptr, *lam_d2 = nullptr;
+    long long d2_stride = 0;
     Chunk *ppchunks = nullptr; int n_ppchunks = 0;    // padded mesh cells
 
     cudaGraphExec_t evolve_exec = nullptr;

@@ -474,18 +474,18 @@ __global__ void k_neg_div(const float *__restrict__ g, int N, float inv_d, int a
 
 // lam_ij products of the second-order source (transpose of Eq. 6's bilinear form).
 __global__ void k_adj_source(const float *__restrict__ lamS, const float *__restrict__ d2, long long n,
-                             float *__restrict__ lam_d2) {
-    // d2: xx, yy, zz, xy, xz, yz (6 x n); lam_d2 same layout
+                             long long stride, float *__restrict__ lam_d2) {
+    // d2: xx, yy, zz, xy, xz, yz (n values each, `stride` apart); lam_d2 same layout
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
          i += (long long)gridDim.x * blockDim.x) {
         const float ls = lamS[i];
-        const float xx = d2[i], yy = d2[n + i], zz = d2[2 * n + i];
+        const float xx = d2[i], yy = d2[stride + i], zz = d2[2 * stride + i];
         lam_d2[i] = ls * (yy + zz);
-        lam_d2[n + i] = ls * (xx + zz);
-        lam_d2[2 * n + i] = ls * (xx + yy);
-        lam_d2[3 * n + i] = -2.0f * ls * d2[3 * n + i];
-        lam_d2[4 * n + i] = -2.0f * ls * d2[4 * n + i];
-        lam_d2[5 * n + i] = -2.0f * ls * d2[5 * n + i];
+        lam_d2[stride + i] = ls * (xx + zz);
+        lam_d2[2 * stride + i] = ls * (xx + yy);
+        lam_d2[3 * stride + i] = -2.0f * ls * d2[3 * stride + i];
+        lam_d2[4 * stride + i] = -2.0f * ls * d2[4 * stride + i];
+        lam_d2[5 * stride + i] = -2.0f * ls * d2[5 * stride + i];
     }
 }
 
@@ -608,7 +608,7 @@ cudaError_t launch_neg_div(Ctx &c, const float *g, int accumulate, float *out) {
 }
 
 cudaError_t launch_adj_source(Ctx &c, const float *lamS, const float *d2, float *lam_d2) {
-    k_adj_source<<<grid_for(c.N3, 256), 256, 0, c.stream>>>(lamS, d2, c.N3, lam_d2);
+    k_adj_source<<<grid_for(c.N3, 256), 256, 0, c.stream>>>(lamS, d2, c.N3, c.d2_stride, lam_d2);
     ++c.launches;
     return cudaGetLastError();
 }
