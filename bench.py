@@ -400,15 +400,24 @@ def study_cost(sc, torch, kw, W, steps, peaks):
 
 
 # ----------------------------------------------------------------------------- roofline
-def kernel_roofline(kt, kw, clocks, peaks, form, box_frac=1.0):
+def solves_x_by_elimination(kw, form):
+    """Whether a Poisson form solves the x axis by elimination: at FDA order 2 the tensor-core forms,
+    and the dense FP32 form where every mesh has at most 128 cells a side."""
+    if kw.get("fda_order", 2) != 2:
+        return False
+    return form in ("tc", "tc4", "tc3") or (form == "simt" and max(box_sizes(kw)[1]) <= 128)
+
+
+def kernel_roofline(kt, kw, clocks, peaks, form, box_frac=1.0, x_elimination=None):
     """Algorithmic bytes or flops per launch of each kernel class and the dominant one.
 
     FP32 form: dense products on CUDA cores (ALU bound, 2 Ng flops per cell per transform):
-    five passes, pass 3 with two transforms, or where passes 4 and 5 are empty, two plane
-    passes of two transforms around the elimination along x (HBM bound).  Tensor-core and
-    radix forms: three, five or six passes, each streaming its mesh once (HBM bound: 4 B read
-    + 4 B written per cell).  Deposit: the positions once (12 B per particle) and the
-    Poisson source written once (4 B per cell).
+    five passes, pass 3 with two transforms, or two plane passes of two transforms around the
+    elimination along x (HBM bound).  Tensor-core and radix forms: three, five or six passes,
+    each streaming its mesh once (HBM bound: 4 B read + 4 B written per cell).  Deposit: the
+    positions once (12 B per particle) and the Poisson source written once (4 B per cell).
+    x_elimination: whether the x axis is solved by elimination (solves_x_by_elimination); None:
+    where the passes that it leaves empty take no time.
     """
     nsc, ng = box_sizes(kw)
     # box_frac: the share of the boxes one launch processes (streamed batches: one batch)
@@ -431,12 +440,12 @@ def kernel_roofline(kt, kw, clocks, peaks, form, box_frac=1.0):
         # streaming its mesh once
         names = ["dst_1_z_fwd", "dst_2_y_fwd", "dst_3_x_fwd_div", "dst_4_z_inv", "dst_5_y_inv",
                  "dst_6_x_inv"]
-        if form != "radix" and kt["dst_6"] < 0.5 * kt["dst_1"]:
+        if form != "radix" and (kt["dst_6"] == 0.0 if x_elimination is None else x_elimination):
             names = names[:2] + ["dst_3_x_elimination"] + names[3:5] + [None]
         for nm in names:
             if nm:
                 work[nm] = ("hbm", 8.0 * M)
-    elif kt["dst_4"] < 0.5 * kt["dst_1"]:
+    elif kt["dst_4"] == 0.0 if x_elimination is None else x_elimination:
         names = ["dst_1_plane_fwd", "dst_2_x_elimination", "dst_3_plane_inv", None, None, None]
         work.update({names[0]: ("alu", 2 * dense), names[1]: ("hbm", 8.0 * M), names[2]: ("alu", 2 * dense)})
     else:
@@ -649,7 +658,7 @@ def run_gpu(args, rank, world, local_rank):
     sc.scola_set_profiling(sim.ctx, False)
     st = sim.stats()
     box_frac = st["batch_boxes"] / st["nboxes"] if st["batches"] > 1 else 1.0
-    dom, rows = kernel_roofline(kt, kw, clk, peaks, args.dst, box_frac)
+    dom, rows = kernel_roofline(kt, kw, clk, peaks, args.dst, box_frac, solves_x_by_elimination(kw, args.dst))
     sc.scola_device_status(sim.ctx)
     d = rows[dom]
     # ncu DRAM bytes per evaluation, keyed by class (dst_i: the i-th pass)
