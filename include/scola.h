@@ -79,7 +79,10 @@ typedef enum scola_dst_variant {
                                     form, timed once on the context's boxes before the first
                                     evolution (where Ng > 222 excludes the dense FP32 form: the
                                     one-axis tensor-core form alone; where Ng > 240 excludes the
-                                    tensor cores: the radix form) */
+                                    tensor cores: the radix form).  The forms differ in rounding
+                                    error, all far inside the tests' bounds: a caller who wants
+                                    the FP32 forms' (RMS force error ~3.5e-6 on 150^3 cells, one
+                                    axis a tensor-core pass ~6e-6) asks for one of them */
 } scola_dst_variant;
 
 typedef enum scola_deposit_form {

@@ -192,7 +192,8 @@ k_box_ids(const BoxDesc *__restrict__ boxes, const Chunk *__restrict__ chunks, i
 }
 
 // (256^3 particles at a = 1: 472 us, 486 us with a remainder per corner index and eight atomics a
-// particle: the L2 rate of the 64-bit atomics, 2.8e11 a second, sets the pace.)
+// particle.  The reductions' requests to L2 set the pace, 1.34e8 of them at 2.8e11 a second: L2 tag
+// stage 76 % of its peak, the SMs' request ports up to 91 %, DRAM 12 % (442 MB).)
 __global__ void k_density_deposit(const float *__restrict__ x, long long n, int N, float inv_d,
                                   unsigned long long *__restrict__ acc) {
     // (whole warps: the deposit shares weights between lanes)

@@ -23,8 +23,9 @@
 // boxes at a time and walks the boxes of its column tile; the pivots depend on the column alone
 // and are computed once per tile.  y waits in shared memory for the backward recursion (this is
 // what bounds the resident threads), the next rows of f, also those of the next boxes, are in
-// flight in registers: 8 rows up to Ng = 128 (3 CTAs of 256 threads an SM at Ng = 96), 16 above,
-// where fewer threads fit (192^3: 290 us with 8 rows, 214 us with 16; 96^3: 106 us and 112 us).  Bound: HBM, 8 bytes a cell.
+// flight in registers: 8 rows up to Ng = 128 (two CTAs of 512 threads an SM for four or more boxes
+// of 96^3), 16 above, where fewer threads fit (16 boxes of 192^3: 290 us with 8 rows, 214 us with
+// 16; 64 of 96^3: 106 us and 112 us).  Bound: HBM, 8 bytes a cell.
 #include <algorithm>
 #include <cstring>
 #include <vector>
@@ -204,8 +205,8 @@ cudaError_t launch_tri_pass(Ctx &c, float *mesh) {
             ngmax = std::max(ngmax, P.Ng);
             nbmax = std::max(nbmax, P.nboxes);
         }
-        // boxes side by side in a CTA: the number that keeps most threads resident per SM (96^3
-        // meshes: 2 boxes, 3 CTAs; 192^3: 4 boxes, 1 CTA)
+        // boxes side by side in a CTA: the number that keeps most threads resident per SM (four boxes
+        // or more of 96^3: 4, in 2 CTAs; of 192^3: 4, in 1 CTA; two or three of 96^3: 2, in 3 CTAs)
         int parts = 1, ctas = 1;
         for (int p = 1; p <= kTriParts && p <= nbmax; ++p) {
             const int n = std::min(16 / p, (int)(kTriSmem / (tri_smem(ngmax, p) + 1024)));

@@ -206,8 +206,9 @@ k_dst(const BoxDesc *__restrict__ boxes, const DstTable *__restrict__ tables,
 // Ng + N_ghost - 1] and the lower corner capped at Ng + N_ghost - 2 (the gradient exists on
 // the grid padded by N_ghost, Sec. 3.4.2).
 //
-// The 32 gathers of order 2 are bound by the L1's wavefronts (78 % of their peak rate at 64 boxes
-// of 96^3 cells, DRAM 21 %): neighbouring particles drift to other rows and lines.  Where the box
+// The 32 gathers of order 2 are bound by the L1's wavefronts (as plain loads, at 64 boxes of 96^3
+// cells: 78 % of their peak rate in k_interp with DRAM at 21 %, 72 % in k_kick_drift with DRAM at
+// 37 %): neighbouring particles drift to other rows and lines.  Where the box
 // has a texture of its padded potential (kTex), 24 of the 32 values come as six 2 x 2 gathers in
 // the (x, z) plane through the texture pipe, which runs beside the load pipe; the eight outer z
 // values stay plain loads (texture gathers alone saturate at 16 cycles a warp instruction).  Force
