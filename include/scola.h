@@ -56,8 +56,9 @@ typedef enum scola_dst_variant {
                                     Ng <= 128 whole x planes in shared memory (z and y in one pass)
                                     and elimination along x */
     SCOLA_DST_TC_3XTF32 = 1,     /* the same products on tcgen05 tensor cores, 3xTF32 split;
-                                    every 2 <= Ng <= 240 (the sine matrix resident in shared
-                                    memory, folded by its mirror symmetry for Ng > 128).  At FDA
+                                    every 2 <= Ng <= 240 but 121 .. 128 (the sine matrix resident in
+                                    shared memory, folded by its mirror symmetry for Ng > 128, beside
+                                    two data stages).  At FDA
                                     order 2 the x axis is solved by elimination: with z and y in
                                     sine space the Laplacian is tridiagonal along x */
     SCOLA_DST_TC_4XTF32 = 3,     /* as 1, plus the lo x lo product (four TF32 products) */
@@ -78,7 +79,7 @@ typedef enum scola_dst_variant {
                                     where every Ng allows it), the dense FP32 form and the radix
                                     form, timed once on the context's boxes before the first
                                     evolution (where Ng > 222 excludes the dense FP32 form: the
-                                    one-axis tensor-core form alone; where Ng > 240 excludes the
+                                    one-axis tensor-core form alone; where some Ng excludes the
                                     tensor cores: the radix form).  The forms differ in rounding
                                     error, all far inside the tests' bounds: a caller who wants
                                     the FP32 forms' (RMS force error ~3.5e-6 on 150^3 cells, one

@@ -178,7 +178,7 @@ scola_status validate(const scola_params *p, std::vector<int32_t> &bufs, std::ve
             return SCOLA_ERR_UNSUPPORTED;
         }
         if (for_kernels && tc_form && !tc_supported(ng)) {
-            set_error("the tensor-core DST needs 2 <= Ng <= 240 (its sine matrix and two data stages in 227 KB of "
+            set_error("the tensor-core DST needs 2 <= Ng <= 240, not 121 .. 128 (its sine matrix and two data stages in 227 KB of "
                       "shared memory)");
             return SCOLA_ERR_UNSUPPORTED;
         }
@@ -822,7 +822,7 @@ scola_status build(scola_ctx *c, const std::vector<BoxGeom> &all_geo) {
     // the radix form: requested, or one more autotuner candidate where every Ng allows it
     bool all_rx = true;
     for (auto &kv : c->tbl_of) all_rx = all_rx && rx_supported(kv.first);
-    // (AUTO where some Ng exceeds the tensor-core form's 240: the radix form, which takes 256)
+    // (AUTO where some Ng excludes the tensor-core form (121 .. 128, > 240): the radix form, which takes 256)
     c->rx = p.dst_variant == SCOLA_DST_RADIX || (p.dst_variant == SCOLA_DST_AUTO && !all_tc && all_rx);
     c->rx_ok = c->rx || (c->dst_auto && all_rx);
     if (c->rx_ok)
